@@ -39,10 +39,10 @@
 // accumulate in the lane's registers (double-float; A_i = -S_i - B_i by
 // translation invariance), the row sums P_j are warp-reduced and kept as one
 // double-float partial per warp in shared memory, summed at the end
-// (n <= kPartialsN).  Larger airfoils take k_adjoint_df_split: the panels are
-// cut into chunks of 256, one block per (airfoil, chunk), and every term of the
-// formula above is added into the caller's gradient buffer by FP64 atomics
-// once per row window, column or node (a few per pair row, not per pair).
+// (n <= kPartialsN).  Larger airfoils and small batches take k_adjoint_df_split:
+// one block per (airfoil, 64 panels, range of rows), every term of the formula
+// above added into the caller's gradient buffer by FP64 atomics once per row
+// window, column or node (a few per pair row, not per pair).
 #include "panel_common.cuh"
 #include "panel_df.cuh"
 
@@ -359,58 +359,92 @@ __global__ void __launch_bounds__(256) k_adjoint_df(
 }
 
 // ---------------------------------------------------------------------------
-// Large airfoils (n > kPartialsN): block (x, y) takes the panels [256 y,
-// 256 y + 256) of airfoil order[x] -- one 32-column block per warp -- against
-// every control point.  Shared memory holds the control points of all rows,
-// lambda, and the constants of the block's own panels only.  Rows are swept in
-// windows of 32: each warp leaves its warp-reduced P_j partials in shared
-// memory, one warp sums the eight and adds lambda_j P_j / 2 to nodes j and
-// j + 1 of the gradient.  The caller's gradient rows are set to zero (or NaN for
-// a failed airfoil) by k_adjoint_prepare first; every contribution goes in by
-// an FP64 atomic add, so the summation order, and the last bits, vary between
-// runs.
+// Large airfoils and small batches (adjoint_split): block (x, y, z) takes the
+// panels [C y, C y + C) of airfoil order[x], C = blockDim.x -- one 32-column
+// block per warp -- against the control points [R z, R z + R), R a multiple of
+// 4.  Shared memory holds the constants of the block's own panels and a window
+// of at most 32 rows (control points, lambda).  Per window each warp leaves its
+// warp-reduced P_j partials in shared memory, one warp sums them and adds
+// lambda_j P_j / 2 to nodes j and j + 1 of the gradient.  k_adjoint_prepare
+// first writes the terms that need no pair sums (or NaN for a failed airfoil);
+// every contribution goes in by an FP64 atomic add, so the summation order, and
+// the last bits, vary between runs.
+//
+// One airfoil is n^2 independent pairs of ~600 instructions: a block for all of
+// its rows keeps one SM busy and 151 idle when the batch is small.  The
+// launcher therefore cuts rows until the chip is full (split_rows).
 // ---------------------------------------------------------------------------
-constexpr int kSplitChunk = 256;
+constexpr int kSplitCols = 64;  // columns and threads per block
 
-__global__ void k_adjoint_prepare(Batch bt, double* __restrict__ grad,
-                                  const int32_t* __restrict__ info) {
-  const int b = bt.order[blockIdx.x];
-  const int n = airfoil_n(bt, b);
-  const bool bad = (info && info[b] != 0) || n > bt.n_max || n < 3;
-  double* gout = grad + 2 * bt.node_off[b];
-  for (int k = threadIdx.x; k < 2 * n; k += blockDim.x) gout[k] = bad ? nan("") : 0.0;
-}
-
-__global__ void __launch_bounds__(256) k_adjoint_df_split(
+__global__ void __launch_bounds__(256) k_adjoint_prepare(
     Batch bt, const double* __restrict__ u, const double* __restrict__ lambda,
     const double* __restrict__ alpha, const double* __restrict__ vinf,
     const double* __restrict__ chord, const double* __restrict__ grad_cl,
     double* __restrict__ grad, const int32_t* __restrict__ info, int lam_weighted) {
+  const int b = bt.order[blockIdx.x];
+  const int n = airfoil_n(bt, b);
+  const bool bad = (info && info[b] != 0) || n > bt.n_max || n < 3;
+  double* gout = grad + 2 * bt.node_off[b];
+  const int k = blockIdx.y * blockDim.x + threadIdx.x;
+  if (k >= n) {
+    // a failed airfoil may have more nodes than the launch's bound covers
+    if (!bad) return;
+  }
+  if (bad) {
+    for (int q = k; q < n; q += gridDim.y * blockDim.x) gout[2 * q] = gout[2 * q + 1] = nan("");
+    return;
+  }
+  const double* nodes = bt.nodes + 2 * bt.node_off[b];
+  const double* ub = u + vec_off(bt, b);
+  const double* lb = lambda + vec_off(bt, b);
+  const double v = vinf ? vinf[b] : 1.0, c = chord ? chord[b] : 1.0;
+  // se scales the explicit dCl/dx term, sl the lambda terms (as in k_adjoint_df)
+  const double se = grad_cl ? grad_cl[b] : (lam_weighted ? 0.0 : 1.0);
+  const double sl = lam_weighted ? 1.0 : se;
+  const double ca = cos(alpha[b]), sa = sin(alpha[b]);
+  const int km = (k == 0) ? n - 1 : k - 1;
+  const int k1 = (k + 1 == n) ? 0 : k + 1;
+  const double hkx = nodes[2 * k1] - nodes[2 * k], hky = nodes[2 * k1 + 1] - nodes[2 * k + 1];
+  const double hmx = nodes[2 * k] - nodes[2 * km], hmy = nodes[2 * k + 1] - nodes[2 * km + 1];
+  const double Lk = sqrt(hkx * hkx + hky * hky), Lm = sqrt(hmx * hmx + hmy * hmy);
+  const double ex = 2.0 / (v * c) * (ub[km] * hmx / Lm - ub[k] * hkx / Lk);
+  const double ey = 2.0 / (v * c) * (ub[km] * hmy / Lm - ub[k] * hky / Lk);
+  const double bx = 0.5 * v * (-sa) * (lb[km] + lb[k]);
+  const double by = 0.5 * v * ca * (lb[km] + lb[k]);
+  gout[2 * k] = se * ex + sl * bx;
+  gout[2 * k + 1] = se * ey + sl * by;
+}
+
+__global__ void __launch_bounds__(kSplitCols) k_adjoint_df_split(
+    Batch bt, const double* __restrict__ u, const double* __restrict__ lambda,
+    const double* __restrict__ grad_cl, double* __restrict__ grad,
+    const int32_t* __restrict__ info, int lam_weighted, int rows) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int ld = bt.n_max;
+  constexpr int ld = kSplitCols, nw = kSplitCols / 32;
   float4* tlog = reinterpret_cast<float4*>(smraw);        // 257
   float2* tatan = reinterpret_cast<float2*>(tlog + 257);  // 34
-  float4* win = reinterpret_cast<float4*>(tatan + 34);    // 8 warps x 32 rows
-  // the current window's 32 rows, two buffers: control points (6 split
+  float4* win = reinterpret_cast<float4*>(tatan + 34);    // nw warps x 32 rows
+  // the current window's rows, two buffers: control points (6 split
   // coordinates, stride 32) and lambda as a float pair
-  float* wrow = reinterpret_cast<float*>(win + 8 * 32);   // 2 x 8 x 32
-  float* cpc = wrow + 2 * 8 * 32;                         // kPanelFields * kSplitChunk
+  float* wrow = reinterpret_cast<float*>(win + nw * 32);  // 2 x 8 x 32
+  float* cpc = wrow + 2 * 8 * 32;                         // kPanelFields * ld
 
   const int b = bt.order[blockIdx.x];
   const int n = airfoil_n(bt, b);
-  const int i0 = blockIdx.y * kSplitChunk;
-  if ((info && info[b] != 0) || n > ld || n < 3 || i0 >= n) return;
+  const int i0 = blockIdx.y * ld;
+  const int jbeg = blockIdx.z * rows, jend = min(n, jbeg + rows);
+  if ((info && info[b] != 0) || n > bt.n_max || n < 3 || i0 >= n || jbeg >= n) return;
   const double* nodes = bt.nodes + 2 * bt.node_off[b];
   const double* ub = u + vec_off(bt, b);
   const double* lb = lambda + vec_off(bt, b);
   double* gout = grad + 2 * bt.node_off[b];
-  const int nc = min(kSplitChunk, n - i0);
+  const int nc = min(ld, n - i0);
   df_stage_tables(tlog, tatan);
-  // the rows of window j0 into buffer (j0 / 32) & 1, a thread per row
+  // the rows of window j0 into its buffer, a thread per row
   auto stage_rows = [&](int j0) {
     const int t = threadIdx.x, k = j0 + t;
-    if (t < 32 && k < n) {
-      float* w = wrow + ((j0 >> 5) & 1) * 256;
+    if (t < 32 && k < jend) {
+      float* w = wrow + (((j0 - jbeg) >> 5) & 1) * 256;
       const int k1 = (k + 1 == n) ? 0 : k + 1;
       const point3 c = make_point(0.5 * (nodes[2 * k] + nodes[2 * k1]),
                                   0.5 * (nodes[2 * k + 1] + nodes[2 * k1 + 1]));
@@ -427,13 +461,10 @@ __global__ void __launch_bounds__(256) k_adjoint_df_split(
   };
   for (int k = threadIdx.x; k < nc; k += blockDim.x) {
     const int i = i0 + k, i1 = (i + 1 == n) ? 0 : i + 1;
-    panel_constants(cpc, kSplitChunk, k, nodes[2 * i], nodes[2 * i + 1], nodes[2 * i1],
+    panel_constants(cpc, ld, k, nodes[2 * i], nodes[2 * i + 1], nodes[2 * i1],
                     nodes[2 * i1 + 1]);
   }
-  const double v = vinf ? vinf[b] : 1.0, c = chord ? chord[b] : 1.0;
-  // se scales the explicit dCl/dx term, sl the lambda terms (as in k_adjoint_df)
-  const double se = grad_cl ? grad_cl[b] : (lam_weighted ? 0.0 : 1.0);
-  const double sl = lam_weighted ? 1.0 : se;
+  const double sl = (grad_cl && !lam_weighted) ? grad_cl[b] : 1.0;
   const double w2pi = sl * kInvTwoPi;
   __syncthreads();
 
@@ -445,11 +476,11 @@ __global__ void __launch_bounds__(256) k_adjoint_df_split(
   const int ic = ok ? il : 0;
   const df2 ui = ok ? df_from_double(ub[i]) : mkdf(0.0f);
   df2 sSx = mkdf(0.0f), sSy = mkdf(0.0f), sKr = mkdf(0.0f), sKi = mkdf(0.0f);
-  for (int j0 = 0; j0 < n; j0 += 32) {
-    const int jn = min(32, n - j0);
+  for (int j0 = jbeg; j0 < jend; j0 += 32) {
+    const int jn = min(32, jend - j0);
     stage_rows(j0);
     __syncthreads();
-    const float* wr = wrow + ((j0 >> 5) & 1) * 256;
+    const float* wr = wrow + (((j0 - jbeg) >> 5) & 1) * 256;
     if (warp_on) {
       df2 rx[4], ry[4];
       for (int t0 = 0; t0 < jn; t0 += 4) {
@@ -460,7 +491,7 @@ __global__ void __launch_bounds__(256) k_adjoint_df_split(
           if (t < jn) {
             const point3 pj = load_point(wr, 32, t);
             df2 gpx, gpy, kr, ki;
-            panel_dG_df(pj, cpc, kSplitChunk, ic, ok && i == j, tlog, tatan, gpx, gpy, kr, ki);
+            panel_dG_df(pj, cpc, ld, ic, ok && i == j, tlog, tatan, gpx, gpy, kr, ki);
             const df2 lj = mkdf(wr[6 * 32 + t], wr[7 * 32 + t]);
             acc_add_prod(sSx, lj, gpx);
             acc_add_prod(sSy, lj, gpy);
@@ -488,8 +519,7 @@ __global__ void __launch_bounds__(256) k_adjoint_df_split(
     __syncthreads();
     if (warp == 0 && lane < jn) {
       df2 sx = mkdf(0.0f), sy = mkdf(0.0f);
-#pragma unroll
-      for (int w = 0; w < 8; ++w) {
+      for (int w = 0; w < nw; ++w) {
         const float4 q = win[w * 32 + lane];
         sx = df_add(sx, mkdf(q.x, q.y));
         sy = df_add(sy, mkdf(q.z, q.w));
@@ -520,29 +550,40 @@ __global__ void __launch_bounds__(256) k_adjoint_df_split(
     atomicAdd(&gout[2 * i1], f * bx);
     atomicAdd(&gout[2 * i1 + 1], f * by);
   }
-  if (blockIdx.y == 0) {
-    // the terms that need no pair sums, once per node
-    const double ca = cos(alpha[b]), sa = sin(alpha[b]);
-    for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      const int km = (k == 0) ? n - 1 : k - 1;
-      const int k1 = (k + 1 == n) ? 0 : k + 1;
-      const double hkx = nodes[2 * k1] - nodes[2 * k], hky = nodes[2 * k1 + 1] - nodes[2 * k + 1];
-      const double hmx = nodes[2 * k] - nodes[2 * km], hmy = nodes[2 * k + 1] - nodes[2 * km + 1];
-      const double Lk = sqrt(hkx * hkx + hky * hky), Lm = sqrt(hmx * hmx + hmy * hmy);
-      const double ex = 2.0 / (v * c) * (ub[km] * hmx / Lm - ub[k] * hkx / Lk);
-      const double ey = 2.0 / (v * c) * (ub[km] * hmy / Lm - ub[k] * hky / Lk);
-      const double bx = 0.5 * v * (-sa) * (lb[km] + lb[k]);
-      const double by = 0.5 * v * ca * (lb[km] + lb[k]);
-      atomicAdd(&gout[2 * k], se * ex + sl * bx);
-      atomicAdd(&gout[2 * k + 1], se * ey + sl * by);
-    }
-  }
+}
+
+static size_t adjoint_split_smem() {
+  return 257 * 16 + 34 * 8 + (size_t)kSplitCols * 16 + 2 * 8 * 32 * 4 +
+         (size_t)kPanelFields * kSplitCols * 4;
+}
+
+// Rows per block of k_adjoint_df_split.  Blocks of 64 columns (12 on an SM at 80
+// registers) waste the fewest lanes and warps on ragged widths: 1216 airfoils of
+// 300 panels took 2937 us in 256-column blocks and take 2278 us, 304 of 1024..2048
+// 11975 -> 10753 us.  256 rows keep a block's prologue below 10 % of its pairs
+// and its share of the last wave small (304 of 1024..2048: 11724 us at all rows,
+// 11096 / 10847 / 10753 us in 2 / 4 / 8 parts); fewer, down to 4, when that
+// leaves less than one wave of blocks (64 of 512: 633 us in 256 x 512 blocks, 405
+// us at 64 x 128; one of 1024: 1032 -> 70 us).
+constexpr int kSplitRows = 256;
+static int split_rows(int B, int n_max) {
+  const int sms = sm_count() > 0 ? sm_count() : 1;
+  const long long wave = 12ll * sms;
+  const long long blocks = (long long)B * ((n_max + kSplitCols - 1) / kSplitCols);
+  const long long z = max((wave + blocks - 1) / blocks, (long long)(n_max + kSplitRows - 1) / kSplitRows);
+  return max(4, (int)((((n_max + z - 1) / z) + 3) & ~3ll));
+}
+
+// Up to kPartialsN panels a block per airfoil is the faster form once the
+// airfoils' 32-column warps fill eight warps on every SM (200 panels, us: 64
+// airfoils 239 against 138 split, 152: 238 / 246, 608: 611 / 742); below it the
+// split fills the chip (100 panels: 64 airfoils 145 -> 68, 304: 170 / 172).
+static bool adjoint_split(int B, int n_max) {
+  return n_max > kPartialsN || (long long)B * ((n_max + 31) / 32) < 8ll * sm_count();
 }
 
 size_t adjoint_df_smem(int n_max) {
-  if (n_max > kPartialsN)
-    return 257 * 16 + 34 * 8 + 8 * 32 * 16 + 2 * 8 * 32 * 4 +
-           (size_t)kPanelFields * kSplitChunk * 4;
+  if (n_max > kPartialsN) return adjoint_split_smem();
   return 257 * 16 + 34 * 8 + (size_t)n_max * 8 * 8 + (size_t)n_max * 4 * 2 +
          (size_t)kPanelFields * n_max * 4 + (size_t)8 * n_max * 16;
 }
@@ -551,20 +592,25 @@ cudaError_t launch_adjoint_df(const Batch& bt, const double* u, const double* la
                               const double* alpha, const double* vinf, const double* chord,
                               const double* grad_cl, double* grad, const int32_t* info,
                               cudaStream_t s, bool lam_weighted) {
-  const size_t smem = adjoint_df_smem(bt.n_max);
   cudaError_t e;
-  if (bt.n_max <= kPartialsN) {
+  if (!adjoint_split(bt.B, bt.n_max)) {
+    const size_t smem = adjoint_df_smem(bt.n_max);
     e = ensure_smem(k_adjoint_df, smem);
     if (e != cudaSuccess) return e;
     k_adjoint_df<<<bt.B, 256, smem, s>>>(bt, u, lambda, alpha, vinf, chord, grad_cl, grad, info,
                                          lam_weighted ? 1 : 0);
   } else {
+    const int rows = split_rows(bt.B, bt.n_max);
+    const size_t smem = adjoint_split_smem();
     e = ensure_smem(k_adjoint_df_split, smem);
     if (e != cudaSuccess) return e;
-    k_adjoint_prepare<<<bt.B, 256, 0, s>>>(bt, grad, info);
-    const dim3 grid(bt.B, (bt.n_max + kSplitChunk - 1) / kSplitChunk);
-    k_adjoint_df_split<<<grid, 256, smem, s>>>(bt, u, lambda, alpha, vinf, chord, grad_cl, grad,
-                                               info, lam_weighted ? 1 : 0);
+    k_adjoint_prepare<<<dim3(bt.B, (bt.n_max + 255) / 256), 256, 0, s>>>(
+        bt, u, lambda, alpha, vinf, chord, grad_cl, grad, info, lam_weighted ? 1 : 0);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    const dim3 grid(bt.B, (bt.n_max + kSplitCols - 1) / kSplitCols, (bt.n_max + rows - 1) / rows);
+    k_adjoint_df_split<<<grid, kSplitCols, smem, s>>>(bt, u, lambda, grad_cl, grad, info,
+                                                      lam_weighted ? 1 : 0, rows);
   }
   return cudaGetLastError();
 }

@@ -327,8 +327,10 @@ class PanelBatch:
         for m > 640 with T 128-column blocks, the step-synchronous LU: the tiled
         copy, T diagonal LUs, one CUDA-core and T - 1 tensor-core triangular
         solves, T - 1 updates, the untranspose of the U tiles and the inversion
-        of the diagonal blocks; the adjoint of n > 256 adds a zeroing launch."""
+        of the diagonal blocks; the split adjoint (n > 256, or fewer 32-column warps
+        than eight per SM) adds a launch for the terms without pair sums."""
         n = 1  # forces
+        sms = torch.cuda.get_device_properties(self.device).multi_processor_count
         for k, (start, cnt, nmax) in enumerate(self.buckets):
             m = nmax + 1
             n += 1  # assemble
@@ -344,7 +346,8 @@ class PanelBatch:
             else:
                 n += 1
             if with_grad:
-                n += 1 + (nmax > 256 and self.flags == bd.PANEL_MIXED)
+                split = nmax > 256 or cnt * (-(-nmax // 32)) < 8 * sms
+                n += 1 + (split and self.flags == bd.PANEL_MIXED)
         return n
 
     # -- autotuning and graph capture -------------------------------------------
