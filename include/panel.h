@@ -110,10 +110,10 @@ typedef enum {
  *     sharing the far field's orientation-free terms.  All give the same
  *     matrix.
  *   PANEL_TUNE_LU(k), k = 1..2: the FP32 LU (panel_solve, PANEL_MIXED, without
- *     PANEL_INVERSE) of airfoils with n_b < 224 keeps the trailing matrix in
+ *     PANEL_INVERSE) of airfoils with n_b < 222 keeps the trailing matrix in
  *     the LU buffer through L2, several airfoils per SM (1), or the whole
- *     matrix in shared memory, one airfoil per SM (2, the choice by size).
- *     The two compute the same factor (the same operations in the same order).
+ *     matrix in shared memory (2); 0 chooses by size and batch.  The two compute
+ *     the same factor (the same operations in the same order).
  * Other values are rejected (PANEL_EINVAL). */
 #define PANEL_TUNE_IR_SHIFT 8
 #define PANEL_TUNE_ROUNDS_SHIFT 12

@@ -46,7 +46,7 @@ def PANEL_TUNE_ROUNDS(sel: int) -> int:
 
 
 def PANEL_TUNE_LU(kind: int) -> int:
-    """FP32 LU field of the flags (n_b < 224): 0 by size, 1 trailing matrix
+    """FP32 LU field of the flags (n_b < 222): 0 by size, 1 trailing matrix
     through L2, 2 whole matrix in shared memory."""
     return int(kind) << PANEL_TUNE_LU_SHIFT
 PANEL_N_MAX = 2048

@@ -14,9 +14,10 @@
 // The FP32 factor depends on the size m = n + 1 and the launch's choices:
 //   PANEL_INVERSE, m <= kGjM (288)   explicit inverse by blocked Gauss-Jordan
 //                                    (k_gj_mixed.cu); a correction is one GEMV;
-//   m <= kSmemLuM (224)              k_lu_smem below: LU with the whole matrix in
-//                                    shared memory (by size, PANEL_TUNE_LU(2)),
-//                                    or k_lu_global (PANEL_TUNE_LU(1));
+//   m <= kSmemLuM (222)              k_lu_smem below: LU with the whole matrix in
+//                                    shared memory (PANEL_TUNE_LU(2)), or
+//                                    k_lu_global (PANEL_TUNE_LU(1)); by default
+//                                    by batch and size (lu_kind_by_size);
 //   m <= kLargeM (640)               k_lu_global below: one block per airfoil,
 //                                    blocked right-looking LU, the trailing
 //                                    matrix in the caller's LU buffer through L2;
@@ -41,76 +42,187 @@ namespace panel {
 
 // ---------------------------------------------------------------------------
 // LU with partial pivoting of one kb x kb diagonal block (kb <= 32) by one
-// warp, register-resident: lane r holds row r (x = its NB columns); rows keep
-// their lanes and `pos` tracks their current position, so an exchange of
-// positions q and p is bookkeeping plus one ipiv entry.  The pivot of column
-// q is the largest |x_q| among the rows not yet pivotal (the lowest position
-// among equal maxima).  The loop is not unrolled (the single warp would run
-// thousands of straight-line instructions once each, fetched from beyond the
-// instruction cache); instead the columns rotate through the registers: at
-// step q the current column is x[0], the later ones x[1 .. NB-1-q], and the
-// finished entries of the earlier columns x[NB-q ..]; each step retires x[0]
-// (the multiplier, or the U entry of a pivotal row) to x[NB-1] and shifts the
-// rest down, so every register index is a constant and after NB steps the
-// columns are back in order.  The reciprocal of the pivot is the correctly
-// rounded one (the same value as 1 / p).  ipiv[q] receives base + the position of column
-// q's pivot row.  On return `fz` is 0, or q + 1 for the first exactly zero (or
-// NaN) pivot column q, after which the block is left as it stands.
+// warp, register-resident: lane r holds row r (x = its 32 columns, zero beyond
+// the block); rows keep their lanes and `pos` tracks their current position, so
+// an exchange of positions q and p is bookkeeping plus one ipiv entry.  The
+// pivot of column q is the largest |x_q| (to 2^-18 of it) among the rows not yet
+// pivotal, the lowest row among equals.
+//
+// One warp walks a chain of kb dependent steps, so a step's latency is what
+// counts.  One REDUX finds value and lane of the pivot together (the lane in the
+// low five bits of the key); every lane takes the reciprocal of its own entry
+// while the reduction runs, and the pivot's comes by a shuffle.  The columns
+// rotate down the registers as they are updated (x[0] is the current one), so
+// that the step loop stays rolled with constant register indices; each finished
+// entry goes to the row's own place in `blk`.  Four groups of eight steps
+// narrow the update from 31 to 7 columns.  193 cycles a step (one warp alone);
+// 390 with a vote for the lane, the rounded reciprocal (__frcp_rn, ~190 cycles)
+// and entries kept in registers by selects; 285 with the pivot row broadcast
+// through shared memory; 180 without any pivot search.
+// ipiv[q] receives base + the position of column q's pivot row.  On return `fz`
+// is 0, or q + 1 for the first exactly zero (or NaN) pivot column q, after which
+// the block's contents have no meaning.
 // ---------------------------------------------------------------------------
-template <int NB>
-__device__ __forceinline__ void warp_block_lu(float (&x)[NB], int& pos, bool& done, int& fz,
-                                              int kb, int* ipiv, int base) {
+// 1 / a by one Newton-Raphson step on the hardware approximation.
+__device__ __forceinline__ float rcp_newton(float a) {
+  float r;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return fmaf(r, fmaf(-a, r, 1.0f), r);
+}
+
+template <int W, class Blk>
+__device__ __forceinline__ void warp_block_lu_group(float (&x)[32], const Blk& blk, int& pos,
+                                                    bool& done, int& fz, int kb, int* ipiv,
+                                                    int base) {
   const int lane = threadIdx.x & 31;
-  // every step is straight-line code: the warp-uniform conditions (the step is
-  // inside the block, no zero pivot so far) act as predicates, not branches
 #pragma unroll 1
-  for (int q = 0; q < NB; ++q) {
-    const bool act = q < kb && fz == 0;
-    const float v = (act && !done) ? fabsf(x[0]) : -1.0f;
-    const unsigned key = (v >= 0.0f) ? __float_as_uint(v) + 1u : 0u;  // |x| bits are monotone
+  for (int lq = 0; lq < 8; ++lq) {
+    const int q = 32 - W + lq;
+    const unsigned bits = __float_as_uint(x[0]) & 0x7fffffe0u;  // |x|, monotone
+    const unsigned key = (!done && x[0] == x[0]) ? bits | (31u - lane) : 0u;
+    const float rcp = rcp_newton(x[0]);
     const unsigned mx = __reduce_max_sync(0xffffffffu, key);
-    const bool ok = act && mx > 1u;  // a nonzero pivot (mx <= 1: zero or NaN column)
-    if (act && !ok) fz = q + 1;
-    // the lowest current position among the maxima
-    const unsigned pm = __reduce_min_sync(0xffffffffu, (ok && key == mx) ? (unsigned)pos : 0xffu);
-    const int pl = (__ffs(__ballot_sync(0xffffffffu, ok && key == mx && pos == (int)pm)) - 1) & 31;
-    const int ql = __ffs(__ballot_sync(0xffffffffu, ok && pos == q)) - 1;  // the row now at q
-    if (ok && lane == 0) ipiv[q] = base + (int)pm;
-    if (ok && lane == ql) pos = (int)pm;
-    if (ok && lane == pl) {
-      pos = q;
-      done = true;
-    }
-    const float inv = __frcp_rn(__shfl_sync(0xffffffffu, x[0], pl));
+    const int pl = 31 - (int)(mx & 31u);
+    const bool ok = mx > 31u;  // a nonzero pivot
+    const float inv = __shfl_sync(0xffffffffu, rcp, pl);
     const float l = x[0] * inv;
-    const bool elim = ok && !done;
+    const bool elim = ok && !done && lane != pl;
+    const float le = elim ? l : 0.0f;
+    if (lane < kb && q < kb) blk(lane, q) = elim ? l : x[0];
 #pragma unroll
-    for (int t = 1; t < NB; ++t) {
-      const float uc = __shfl_sync(0xffffffffu, x[t], pl);
-      x[t] = (elim && t < NB - q) ? fmaf(-l, uc, x[t]) : x[t];  // a later column
+    for (int t = 1; t < W; ++t) x[t - 1] = fmaf(-le, __shfl_sync(0xffffffffu, x[t], pl), x[t]);
+    x[W - 1] = 0.0f;
+    // bookkeeping, off the chain
+    const int pm = __shfl_sync(0xffffffffu, pos, pl);
+    if (ok) {
+      if (lane == 0) ipiv[q] = base + pm;
+      if (pos == q) pos = pm;
+      if (lane == pl) {
+        pos = q;
+        done = true;
+      }
+    } else if (q < kb && fz == 0) {
+      fz = q + 1;
     }
-    const float out = elim ? l : x[0];
-#pragma unroll
-    for (int t = 0; t < NB - 1; ++t) x[t] = x[t + 1];
-    x[NB - 1] = out;
   }
+}
+
+template <class Blk>
+__device__ __forceinline__ void warp_block_lu(float (&x)[32], const Blk& blk, int& pos, bool& done,
+                                              int& fz, int kb, int* ipiv, int base) {
+  warp_block_lu_group<32>(x, blk, pos, done, fz, kb, ipiv, base);
+  if (kb > 8) warp_block_lu_group<24>(x, blk, pos, done, fz, kb, ipiv, base);
+  if (kb > 16) warp_block_lu_group<16>(x, blk, pos, done, fz, kb, ipiv, base);
+  if (kb > 24) warp_block_lu_group<8>(x, blk, pos, done, fz, kb, ipiv, base);
+}
+
+// ---------------------------------------------------------------------------
+// The factored diagonal block as the other steps of a panel read it, in shared
+// memory: row q of U and column q of L from the diagonal outwards (u[q][s] =
+// U(q, q + 1 + s), l[q][s] = L(q + 1 + s, q), 0 beyond the block) and the
+// reciprocals of U's diagonal.  A substitution step then reads its 31
+// multipliers as eight broadcast vector loads at the same register indices in
+// every step, so that the step loop stays rolled.
+// ---------------------------------------------------------------------------
+struct alignas(16) DiagTab {
+  float u[32 * 32];
+  float l[32 * 32];
+  float rinv[32];
+  int bperm[32];  // final row q of the block = row bperm[q] before its exchanges
+  int fz;         // 0, or the first zero pivot column + 1
+  int moved;      // some row of the block was exchanged
+  int pad[2];
+};
+
+// LU of the kb x kb diagonal block by the calling warp into the table; blk(r, t)
+// are the block's entries, overwritten.  The pivots go to ipiv[0 .. kb) (+ base).
+template <class Blk>
+__device__ __forceinline__ void diag_lu(const Blk& blk, int kb, int* ipiv, int base, DiagTab& d) {
+  const int lane = threadIdx.x & 31;
+  float x[32];
+#pragma unroll
+  for (int t = 0; t < 32; ++t) x[t] = (lane < kb && t < kb) ? blk(lane, t) : 0.0f;
+  int pos = lane;
+  bool done = lane >= kb;  // already a pivot row (or outside the block)
+  int fz = 0;
+  warp_block_lu(x, blk, pos, done, fz, kb, ipiv, base);
+  // the lane's row sits at `pos` of the block (rows beyond kb: zero, unit pivot)
+  float* ur = d.u + pos * 31 - 1;  // U(pos, t) at ur + pos + t
+  float* lc = d.l + pos - 1;       // L(pos, t) at lc + 31 t
+#pragma unroll 4
+  for (int t = 0; t < 32; ++t) {
+    const float v = (lane < kb && t < kb) ? blk(lane, t) : 0.0f;
+    if (t != pos) *(t > pos ? ur + t : lc + 31 * t) = v;
+  }
+  const float dia = lane < kb ? blk(lane, pos) : 1.0f;
+  d.rinv[pos] = 1.0f / dia;
+  d.bperm[pos] = lane;
+  const bool moved = __any_sync(0xffffffffu, pos != lane);
+  if (lane == 0) {
+    d.fz = fz;
+    d.moved = moved ? 1 : 0;
+  }
+}
+
+// The entries beyond the block's triangles, once per kernel (all threads).
+__device__ __forceinline__ void diag_tab_init(DiagTab& d) {
+  for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x)
+    if ((e & 31) >= 31 - (e >> 5)) d.u[e] = d.l[e] = 0.0f;
+}
+
+// Substitution against the table, right-looking, a right-hand side per thread in
+// x: SCALE, x <- x U^{-1} (a row); else x <- L^{-1} x (a column, unit L).  Each
+// final entry goes to out(q, value).  The entries rotate down the registers as
+// they are updated (x[0] is the current one), in four groups of eight steps
+// whose updates narrow from 31 to 7 entries: 608 multiply-adds a thread for the
+// 496 of the triangle, and a loop body short enough to stay in the instruction
+// cache (the fully unrolled form with one scalar load per multiply-add took
+// 8-12 thousand cycles a panel, bound by its shared-memory loads).
+template <int W, bool SCALE, class Out>
+__device__ __forceinline__ void tri_group(float (&x)[32], const DiagTab& d, const Out& out) {
+#pragma unroll 1
+  for (int lq = 0; lq < 8; ++lq) {
+    const int q = 32 - W + lq;
+    const float4* m = reinterpret_cast<const float4*>((SCALE ? d.u : d.l) + q * 32);
+    const float xq = SCALE ? x[0] * d.rinv[q] : x[0];
+    out(q, xq);
+#pragma unroll
+    for (int t4 = 0; t4 < W / 4; ++t4) {
+      const float4 f = m[t4];
+      x[4 * t4] = fmaf(-xq, f.x, x[4 * t4 + 1]);
+      x[4 * t4 + 1] = fmaf(-xq, f.y, x[4 * t4 + 2]);
+      x[4 * t4 + 2] = fmaf(-xq, f.z, x[4 * t4 + 3]);
+      x[4 * t4 + 3] = (4 * t4 + 4 < W) ? fmaf(-xq, f.w, x[(4 * t4 + 4) & 31]) : 0.0f;
+    }
+  }
+}
+template <bool SCALE, class Out>
+__device__ __forceinline__ void tri_subst(float (&x)[32], const DiagTab& d, const Out& out) {
+  tri_group<32, SCALE>(x, d, out);
+  tri_group<24, SCALE>(x, d, out);
+  tri_group<16, SCALE>(x, d, out);
+  tri_group<8, SCALE>(x, d, out);
 }
 
 // ---------------------------------------------------------------------------
 // The LU kernel, factor in global memory (kSmemLuM < m <= kLargeM, or every
-// m <= kLargeM with PANEL_TUNE_LU(1)): blocked right-looking
-// with the current panel of NB columns staged in shared memory (rows spread
-// over the threads), the row exchanges, U12 and the rank-NB update applied to
-// the factor in the caller's LU buffer through L2.  Shared memory stays small
-// (the panel plus a 128-column slab of U12), so several airfoils share an SM
-// and hide each other's latencies.
+// m <= kLargeM with PANEL_TUNE_LU(1)): blocked right-looking with the current
+// panel of 32 columns staged in shared memory, transposed (panel column q at
+// PT[q ldt + row]: the update reads eight rows' multipliers with two broadcast
+// vector loads), the row exchanges, U12 and the rank-32 update applied to the
+// factor in the caller's LU buffer through L2.  Shared memory stays small (the
+// panel plus a 128-column slab of U12), so several airfoils share an SM and
+// hide each other's latencies.
 // ---------------------------------------------------------------------------
+constexpr int kSlabW = 128;  // columns of U12 staged at a time
+
 // A22 -= L21 U12 over the columns [cc, cc + 32 J) of the staged U12 slab: warp
-// w takes the 8-row tiles w, w + 8, ...; lane l the columns cc + l + 32 j.
-template <int J, int LDP, int CW>
-__device__ __forceinline__ void update_tiles(float* __restrict__ F, const float* __restrict__ P,
-                                             const float* __restrict__ U, int m, int k0, int k1,
-                                             int kb, int cc, int nrt) {
+// w takes the 8-row tiles w, w + 8, ...; lane l the columns cc + l + 32 j.  lt:
+// row k1 of the transposed panel.
+template <int J>
+__device__ __forceinline__ void update_tiles(float* __restrict__ F, const float* __restrict__ lt,
+                                             int ldt, const float* __restrict__ U, int m, int k1,
+                                             int cc, int nrt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int rt = warp; rt < nrt; rt += kWarps) {
     const int r0 = k1 + 8 * rt;
@@ -122,13 +234,15 @@ __device__ __forceinline__ void update_tiles(float* __restrict__ F, const float*
         const int r = r0 + aa, c = cc + lane + 32 * j;
         acc[aa][j] = (r < m && c < m) ? F[r * m + c] : 0.0f;
       }
+    const float* l0 = lt + 8 * rt;
 #pragma unroll 4
-    for (int q = 0; q < kb; ++q) {
-      float lv[8], uv[J];
+    for (int q = 0; q < 32; ++q) {
+      const float4 la = *reinterpret_cast<const float4*>(l0 + q * ldt);
+      const float4 lb = *reinterpret_cast<const float4*>(l0 + q * ldt + 4);
+      const float lv[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
+      float uv[J];
 #pragma unroll
-      for (int aa = 0; aa < 8; ++aa) lv[aa] = (r0 + aa < m) ? P[(r0 + aa - k0) * LDP + q] : 0.0f;
-#pragma unroll
-      for (int j = 0; j < J; ++j) uv[j] = U[q * CW + lane + 32 * j];
+      for (int j = 0; j < J; ++j) uv[j] = U[q * kSlabW + lane + 32 * j];
 #pragma unroll
       for (int aa = 0; aa < 8; ++aa)
 #pragma unroll
@@ -144,11 +258,13 @@ __device__ __forceinline__ void update_tiles(float* __restrict__ F, const float*
   }
 }
 
-template <int NB>
+// Row stride of the transposed panel: rows padded to whole 8-row tiles, and 4
+// mod 32, so that 4 rows x 8 columns moved by a warp touch all banks.
+__host__ __device__ constexpr int lu_panel_ld(int m) { return ((m + 8 + 31) & ~31) + 4; }
+
 __global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int LDP = NB + 1;
-  constexpr int CW = 128;  // GEMM column slab
+  constexpr int NB = 32;
   const Batch& bt = a.bt;
   const int b = bt.order[blockIdx.x];
   const int n = airfoil_n(bt, b);
@@ -162,18 +278,18 @@ __global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
   if (m > kLargeM) return;  // taken by the blocked factor (k_lu_large.cu)
   if (m <= kSmemLuM && a.lu_kind != 1) return;  // taken by k_lu_smem
   const int mv = bt.n_max + 1;
-  float* P = reinterpret_cast<float*>(smraw);           // mv x LDP panel
-  float* U = P + mv * LDP;                              // NB x CW slab of U12
-  double* red = reinterpret_cast<double*>(
-      (reinterpret_cast<uintptr_t>(U + NB * CW) + 15) & ~(uintptr_t)15);  // 32
-  unsigned long long* cand = reinterpret_cast<unsigned long long*>(red + 32);  // kWarps
-  int* ipiv = reinterpret_cast<int*>(cand + kWarps);    // mv
-  int* bperm = ipiv + mv;  // NB: final row q of the block = row k0 + bperm[q] before its exchanges
+  DiagTab& dt = *reinterpret_cast<DiagTab*>(smraw);
+  float* U = reinterpret_cast<float*>(smraw + sizeof(DiagTab));  // NB x kSlabW slab of U12
+  double* red = reinterpret_cast<double*>(U + NB * kSlabW);      // 32
+  float* PT = reinterpret_cast<float*>(red + 32);                // NB x ldt panel, transposed
+  const int ldt = lu_panel_ld(mv);
+  int* ipiv = reinterpret_cast<int*>(PT + NB * ldt);             // mv
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t moff = bt.mat_off[b];
   const float* Ah = a.A_hi + moff;
   float* F = a.LU + moff;
+  diag_tab_init(dt);
   const float sf = (float)border_scale(Ah, n, m, red);
   for (int rr = warp; rr < m; rr += kWarps)
     for (int cc = lane; cc < m; cc += 32) {
@@ -182,175 +298,139 @@ __global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
     }
   __syncthreads();
 
+  const int pc = lane & 7, pr = lane >> 3;  // panel moves: 8 columns x 4 rows per warp
   for (int k0 = 0; k0 < m; k0 += NB) {
     const int kb = min(NB, m - k0);
     const int rows = m - k0;
     // ---- stage the panel ----
-    for (int r = warp; r < rows; r += kWarps)
-      if (lane < kb) P[r * LDP + lane] = F[(k0 + r) * m + k0 + lane];
-    __syncthreads();
-    // ---- factor the panel: LU of the diagonal block by warp 0 (pivot search
-    // inside the block's rows, lane = column), then L21 = A21 U11^{-1} with a
-    // thread per row below the block ----
-    if (warp == 0) {
-      // register-resident: lane r holds row r of the diagonal block (x[t] =
-      // column t); rows keep their lanes and pos tracks their current position,
-      // so an exchange of positions q and p is bookkeeping plus one ipiv entry
-      float x[NB];
+    for (int r = 4 * warp + pr; r < rows; r += 4 * kWarps)
 #pragma unroll
-      for (int t = 0; t < NB; ++t) x[t] = (lane < kb && t < kb) ? P[lane * LDP + t] : 0.0f;
-      int pos = lane;
-      bool done = lane >= kb;  // already a pivot row (or outside the block)
-      int fz = 0;
-      warp_block_lu<NB>(x, pos, done, fz, kb, ipiv + k0, k0);
-      __syncwarp();
-      if (lane < kb) {
-#pragma unroll
-        for (int t = 0; t < NB; ++t)
-          if (t < kb) P[pos * LDP + t] = x[t];
-        bperm[pos] = lane;
+      for (int i = 0; i < 4; ++i) {
+        const int t = 8 * i + pc;
+        if (t < kb) PT[t * ldt + r] = F[(k0 + r) * m + k0 + t];
       }
-      __syncwarp();
-      if (lane == 0) cand[0] = (unsigned long long)fz;
-      if (lane < kb && fz == 0) red[lane] = (double)(1.0f / P[lane * LDP + lane]);
-    }
     __syncthreads();
-    if (cand[0] != 0ull) {
+    // ---- LU of the diagonal block by warp 0 (pivot search inside the block) ----
+    if (warp == 0)
+      diag_lu([&](int r, int t) -> float& { return PT[t * ldt + r]; }, kb, ipiv + k0, k0, dt);
+    __syncthreads();
+    if (dt.fz != 0) {
       if (tid == 0) {
-        a.info[b] = k0 + (int)cand[0];
+        a.info[b] = k0 + dt.fz;
         if (a.iters) a.iters[b] = 0;
       }
       return;
     }
-    if (rows > kb) {  // then kb == NB
-      for (int r = kb + tid; r < rows; r += kThreads) {
-        float x[NB];
-#pragma unroll
-        for (int t = 0; t < NB; ++t) x[t] = P[r * LDP + t];
-        // right-looking: once x_q is final it goes into every later column
-        // (the same terms in the same order as the row's dot products)
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-          x[q] *= (float)red[q];
-#pragma unroll
-          for (int t = q + 1; t < NB; ++t) x[t] = fmaf(-x[q], P[q * LDP + t], x[t]);
-        }
-#pragma unroll
-        for (int t = 0; t < NB; ++t) P[r * LDP + t] = x[t];
-      }
-      __syncthreads();
-    }
-    // ---- write the panel back, exchange rows outside it ----
-    for (int r = warp; r < rows; r += kWarps)
-      if (lane < kb) F[(k0 + r) * m + k0 + lane] = P[r * LDP + lane];
-    // the exchanges of this block's rows: composed into bperm, all loads of a
-    // column in flight at once; the columns right of the panel read their rows
-    // through bperm in the U12 solve below instead
-    for (int c = tid; c < k0; c += kThreads) {
-      float v[NB];
-#pragma unroll
-      for (int q = 0; q < NB; ++q) v[q] = (q < kb) ? F[(k0 + bperm[q]) * m + c] : 0.0f;
-#pragma unroll
-      for (int q = 0; q < NB; ++q)
-        if (q < kb) F[(k0 + q) * m + c] = v[q];
-    }
-    __syncthreads();
     const int k1 = k0 + kb;
-    if (k1 >= m) break;
-    // ---- U12 = L11^{-1} A12, a column per lane, unrolled forward substitution
-    // (here kb == NB: a panel with columns right of it is full) ----
-    for (int cb = k1 + 32 * warp; cb < m; cb += kThreads) {
-      const int c = cb + lane;
-      const bool ok = c < m;
-      float col[NB];
+    // ---- L21 = A21 U11^{-1}, a row per thread, in place in PT; U12 = L11^{-1}
+    // A12, a column per thread, the rows read through the block's exchanges; and
+    // the two inverses of the diagonal block the refinement takes, U11^{-1} as 32
+    // more rows (of the identity) and L11^{-1} as 32 more columns.  A warp takes
+    // 32 rows or columns (rows below the block only beside a full block) ----
+    const int nw = (m - k1 + 31) >> 5;
+    for (int w = warp; w < 2 * nw + 2; w += kWarps) {
+      float x[32];
+      if (w == 0) {
 #pragma unroll
-      for (int t = 0; t < NB; ++t) col[t] = ok ? F[(k0 + bperm[t]) * m + c] : 0.0f;
+        for (int t = 0; t < 32; ++t) x[t] = (t == lane) ? 1.0f : 0.0f;
+        float* G = F + (k0 + lane) * m + k0;
+        tri_subst<true>(x, dt, [&](int q, float v) {
+          if (lane < kb && q < kb && q >= lane) G[q] = v;
+        });
+      } else if (w == 1) {
 #pragma unroll
-      for (int q = 0; q < NB; ++q) {
-        const float x = col[q];
-        if (ok) F[(k0 + q) * m + c] = x;
+        for (int t = 0; t < 32; ++t) x[t] = (t == lane) ? 1.0f : 0.0f;
+        float* G = F + k0 * m + k0 + lane;
+        tri_subst<false>(x, dt, [&](int q, float v) {
+          if (q < kb && q > lane) G[q * m] = v;
+        });
+      } else if (w < 2 + nw) {
+        const int r = kb + 32 * (w - 2) + lane;
+        const bool ok = r < rows;
 #pragma unroll
-        for (int t = q + 1; t < NB; ++t) col[t] = fmaf(-P[t * LDP + q], x, col[t]);
+        for (int t = 0; t < 32; ++t) x[t] = ok ? PT[t * ldt + r] : 0.0f;
+        tri_subst<true>(x, dt, [&](int q, float v) {
+          if (ok) PT[q * ldt + r] = v;
+        });
+      } else {
+        const int c = k1 + 32 * (w - 2 - nw) + lane;
+        const bool ok = c < m;
+#pragma unroll
+        for (int t = 0; t < 32; ++t) x[t] = ok ? F[(k0 + dt.bperm[t]) * m + c] : 0.0f;
+        float* G = F + k0 * m + c;
+        tri_subst<false>(x, dt, [&](int q, float v) {
+          if (ok) G[q * m] = v;
+        });
       }
     }
+    // the exchanges of this block's rows on the columns left of it: composed
+    // into bperm, all loads of a column in flight at once
+    if (dt.moved)
+      for (int c = tid; c < k0; c += kThreads) {
+        float v[NB];
+#pragma unroll
+        for (int q = 0; q < NB; ++q) v[q] = (q < kb) ? F[(k0 + dt.bperm[q]) * m + c] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < NB; ++q)
+          if (q < kb) F[(k0 + q) * m + c] = v[q];
+      }
     __syncthreads();
+    if (k1 >= m) break;
+    // ---- L21 back to the factor ----
+    for (int r = kb + 4 * warp + pr; r < rows; r += 4 * kWarps)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) F[(k0 + r) * m + k0 + 8 * i + pc] = PT[(8 * i + pc) * ldt + r];
     // ---- A22 -= L21 U12, 128-column slabs of U12 staged in shared memory ----
     const int nrt = (m - k1 + 7) >> 3;
-    for (int cc = k1; cc < m; cc += CW) {
+    for (int cc = k1; cc < m; cc += kSlabW) {
       for (int t = warp; t < kb; t += kWarps)
 #pragma unroll
-        for (int j = 0; j < CW / 32; ++j) {
+        for (int j = 0; j < kSlabW / 32; ++j) {
           const int c = cc + lane + 32 * j;
-          U[t * CW + lane + 32 * j] = (c < m) ? F[(k0 + t) * m + c] : 0.0f;
+          U[t * kSlabW + lane + 32 * j] = (c < m) ? F[(k0 + t) * m + c] : 0.0f;
         }
       __syncthreads();
       // register tiles 8 rows x 32 J columns, J = 1..4 by the width of the slab
-      const int J = min(CW / 32, (m - cc + 31) >> 5);
+      const int J = min(kSlabW / 32, (m - cc + 31) >> 5);
       if (J == 4)
-        update_tiles<4, LDP, CW>(F, P, U, m, k0, k1, kb, cc, nrt);
+        update_tiles<4>(F, PT + kb, ldt, U, m, k1, cc, nrt);
       else if (J == 3)
-        update_tiles<3, LDP, CW>(F, P, U, m, k0, k1, kb, cc, nrt);
+        update_tiles<3>(F, PT + kb, ldt, U, m, k1, cc, nrt);
       else if (J == 2)
-        update_tiles<2, LDP, CW>(F, P, U, m, k0, k1, kb, cc, nrt);
+        update_tiles<2>(F, PT + kb, ldt, U, m, k1, cc, nrt);
       else
-        update_tiles<1, LDP, CW>(F, P, U, m, k0, k1, kb, cc, nrt);
+        update_tiles<1>(F, PT + kb, ldt, U, m, k1, cc, nrt);
       __syncthreads();
     }
   }
-  // the diagonal blocks inverted in shared memory (the panel and slab buffers
-  // are free now: a 32 x LDP slot per warp), then written back
-  {
-    float* S = P + warp * (NB * LDP);
-    const int nb = (m + NB - 1) / NB;
-    for (int d = warp; d < nb; d += kWarps) {
-      const int d0 = NB * d, kbd = min(NB, m - d0);
-      for (int r = 0; r < kbd; ++r)
-        if (lane < kbd) S[r * LDP + lane] = F[(d0 + r) * m + d0 + lane];
-      __syncwarp();
-      invert_block(S, LDP, kbd);
-      for (int r = 0; r < kbd; ++r)
-        if (lane < kbd) F[(d0 + r) * m + d0 + lane] = S[r * LDP + lane];
-      __syncwarp();
-    }
-  }
-  __syncthreads();
   int32_t* gpiv = a.piv + vec_off(bt, b);
   for (int k = tid; k < m; k += kThreads) gpiv[k] = ipiv[k];
 }
 
 // ---------------------------------------------------------------------------
 // The LU kernel with the whole matrix in shared memory (3 <= m <= kSmemLuM):
-// one block of 512 threads per airfoil and per SM.  The algorithm and the
-// factor's layout are those of k_lu_global (32-column panels, the pivot search
-// inside the diagonal block, register LU of the diagonal block by one warp, L21
-// by a thread per row, the block's exchanges composed, U12 by a thread per
-// column, the rank-32 update in 8 x 32J register tiles accumulated in the same
-// order, the 32 x 32 diagonal blocks inverted at the end), so the two kernels
-// store the same factor bit for bit.  Here every step works on the scaled
-// matrix staged once in shared memory (odd row stride: conflict-free columns)
-// and the factor goes to the caller's buffer once: one read of the hi plane and
-// one write of the factor per airfoil.  Since one airfoil has the SM to itself,
-// the steps are arranged to keep its warps busy:
-//   A  L21 (threads 0..255, one row each, also kept transposed in LT so that the
-//      update reads eight rows' multipliers with two broadcast vector loads)
-//      and U12 (threads 256..511, one column each) at once, then the exchanges
-//      on the columns left of the panel;
+// one block of NT threads per airfoil.  The algorithm, its operations and their
+// order are those of k_lu_global, so the two kernels store the same factor bit
+// for bit.  Here every step works on the scaled matrix staged once in shared
+// memory (odd row stride: conflict-free columns) and the factor goes to the
+// caller's buffer once: one read of the hi plane and one write of the factor
+// per airfoil.  One (m > 160 or so) or a few airfoils have the SM to themselves,
+// so the steps are arranged to keep the warps busy:
+//   A  the first half of the threads: L21, a row each, also kept transposed in
+//      LT so that the update reads eight rows' multipliers with two broadcast
+//      vector loads, and the rows of U11^{-1}; the second half: U12, a column
+//      each, and the columns of L11^{-1}; the inverses replace the block;
 //   B  the update of the next panel's 32 columns;
-//   C  warp 0 factors the next diagonal block (look-ahead) while warps 1..15
+//   C  warp 0 factors the next diagonal block (look-ahead) while the others
 //      update the remaining columns.
 // ---------------------------------------------------------------------------
-constexpr int kSmemLuThreads = 512;
-constexpr int kSmemLuWarps = kSmemLuThreads / 32;
-static_assert(kSmemLuM <= 256, "k_lu_smem moves rows of at most 8 x 32 columns");
-static_assert(kSmemLuM - 32 <= kSmemLuThreads / 2, "a thread per row / column in phase A");
-
 // A22 -= L21 U12 on rows [r0, r0 + 8) x columns cc + lane + 32 j (j < J): the
 // multipliers of the 8 rows from LT (panel column q at LT[q ldt + r - k1]),
-// U12 from the matrix rows k0..k0 + kb.
+// U12 from the matrix rows k0..k0 + 32.
 template <int J>
 __device__ __forceinline__ void smem_update_tile(float* __restrict__ F, int ld,
                                                  const float* __restrict__ LT, int ldt, int m,
-                                                 int k0, int k1, int kb, int r0, int cc) {
+                                                 int k0, int k1, int r0, int cc) {
   const int lane = threadIdx.x & 31;
   float acc[8][J];
 #pragma unroll
@@ -362,7 +442,7 @@ __device__ __forceinline__ void smem_update_tile(float* __restrict__ F, int ld,
     }
   const float* lt = LT + (r0 - k1);
 #pragma unroll 4
-  for (int q = 0; q < kb; ++q) {
+  for (int q = 0; q < 32; ++q) {
     const float4 la = *reinterpret_cast<const float4*>(lt + q * ldt);
     const float4 lb = *reinterpret_cast<const float4*>(lt + q * ldt + 4);
     const float lv[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
@@ -387,58 +467,34 @@ __device__ __forceinline__ void smem_update_tile(float* __restrict__ F, int ld,
 }
 
 // Update tasks of 8 rows x 32 J columns over the columns [c0, c1) of the rows
-// [k1, m), distributed over the warps w0 .. kSmemLuWarps - 1.
+// [k1, m), shared by the calling warps: the w-th of nw.
 __device__ __forceinline__ void smem_update(float* F, int ld, const float* LT, int ldt, int m,
-                                            int k0, int k1, int kb, int c0, int c1, int w0,
+                                            int k0, int k1, int c0, int c1, int w, int nw,
                                             int cw) {
-  const int warp = threadIdx.x >> 5;
-  if (warp < w0 || c1 <= c0) return;
+  if (c1 <= c0) return;
   const int nrt = (m - k1 + 7) >> 3, ncs = (c1 - c0 + cw - 1) / cw;
-  for (int task = warp - w0; task < nrt * ncs; task += kSmemLuWarps - w0) {
+  for (int task = w; task < nrt * ncs; task += nw) {
     const int r0 = k1 + 8 * (task / ncs), cc = c0 + cw * (task % ncs);
     const int J = min(cw / 32, (min(c1, m) - cc + 31) >> 5);
     if (J >= 4)
-      smem_update_tile<4>(F, ld, LT, ldt, m, k0, k1, kb, r0, cc);
+      smem_update_tile<4>(F, ld, LT, ldt, m, k0, k1, r0, cc);
     else if (J == 3)
-      smem_update_tile<3>(F, ld, LT, ldt, m, k0, k1, kb, r0, cc);
+      smem_update_tile<3>(F, ld, LT, ldt, m, k0, k1, r0, cc);
     else if (J == 2)
-      smem_update_tile<2>(F, ld, LT, ldt, m, k0, k1, kb, r0, cc);
+      smem_update_tile<2>(F, ld, LT, ldt, m, k0, k1, r0, cc);
     else
-      smem_update_tile<1>(F, ld, LT, ldt, m, k0, k1, kb, r0, cc);
+      smem_update_tile<1>(F, ld, LT, ldt, m, k0, k1, r0, cc);
   }
 }
 
-// LU of the diagonal block at (k0, k0), kb x kb, by the calling warp: the block
-// rows in their final order, the pivots in ipiv[k0 ..], the composed exchanges
-// in bperm, 1 / U_tt in red, and in *fz 0 or the first zero pivot column + 1.
-__device__ __forceinline__ void smem_diag_lu(float* F, int ld, int k0, int kb, int* ipiv,
-                                             int* bperm, double* red,
-                                             unsigned long long* fzp) {
-  constexpr int NB = 32;
-  const int lane = threadIdx.x & 31;
-  float* P = F + k0 * ld + k0;
-  float x[NB];
-#pragma unroll
-  for (int t = 0; t < NB; ++t) x[t] = (lane < kb && t < kb) ? P[lane * ld + t] : 0.0f;
-  int pos = lane;
-  bool done = lane >= kb;
-  int fz = 0;
-  warp_block_lu<NB>(x, pos, done, fz, kb, ipiv + k0, k0);
-  __syncwarp();
-  if (lane < kb) {
-#pragma unroll
-    for (int t = 0; t < NB; ++t)
-      if (t < kb) P[pos * ld + t] = x[t];
-    bperm[pos] = lane;
-  }
-  __syncwarp();
-  if (lane == 0) *fzp = (unsigned long long)fz;
-  if (lane < kb && fz == 0) red[lane] = (double)(1.0f / P[lane * ld + lane]);
-}
+// Row stride of the transposed panel: the rows below the first block, in whole
+// 8-row tiles.
+__host__ __device__ constexpr int lu_smem_ldt(int m) { return m > 32 ? (m - 32 + 7) & ~7 : 8; }
 
-__global__ void __launch_bounds__(kSmemLuThreads, 1) k_lu_smem(SolveArgs a) {
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_lu_smem(SolveArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int NB = 32;
+  constexpr int NB = 32, NW = NT / 32;
   const Batch& bt = a.bt;
   const int b = bt.order[blockIdx.x];
   const int n = airfoil_n(bt, b);
@@ -452,145 +508,146 @@ __global__ void __launch_bounds__(kSmemLuThreads, 1) k_lu_smem(SolveArgs a) {
   if (m > kSmemLuM || a.lu_kind == 1) return;  // taken by k_lu_global or the blocked factor
   const int ld = m | 1;
   const int mv = bt.n_max + 1;
-  const int ldv = mv | 1;
-  const int ldt = (mv + 7) & ~7;
-  float* F = reinterpret_cast<float*>(smraw);  // m x ld
-  float* LT = reinterpret_cast<float*>(
-      (reinterpret_cast<uintptr_t>(F + (size_t)mv * ldv) + 15) & ~(uintptr_t)15);  // NB x ldt
-  double* red = reinterpret_cast<double*>(LT + NB * ldt);                          // 32
-  unsigned long long* cand = reinterpret_cast<unsigned long long*>(red + 32);      // 1
-  int* ipiv = reinterpret_cast<int*>(cand + 2);                                    // mv
-  int* bperm = ipiv + mv;                                                          // NB
+  const int ldt = lu_smem_ldt(mv);
+  DiagTab& dt = *reinterpret_cast<DiagTab*>(smraw);
+  double* red = reinterpret_cast<double*>(smraw + sizeof(DiagTab));  // 32
+  float* LT = reinterpret_cast<float*>(red + 32);                    // NB x ldt
+  int* ipiv = reinterpret_cast<int*>(LT + NB * ldt);                 // mv
+  float* F = reinterpret_cast<float*>(ipiv + mv);                    // m x ld
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t moff = bt.mat_off[b];
   const float* Ah = a.A_hi + moff;
   // the hi plane in by asynchronous copies (every element of the thread in
   // flight at once; rows of stride m are only 4-byte aligned), a warp per row
-  for (int rr = warp; rr < m; rr += kSmemLuWarps)
+  for (int rr = warp; rr < m; rr += NW)
     for (int cc = lane; cc < m; cc += 32) {
       const unsigned dst = (unsigned)__cvta_generic_to_shared(F + rr * ld + cc);
       asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(Ah + rr * m + cc)
                    : "memory");
     }
   asm volatile("cp.async.commit_group;\n" ::: "memory");
+  diag_tab_init(dt);
   const float sf = (float)border_scale(Ah, n, m, red);
   asm volatile("cp.async.wait_group 0;\n" ::: "memory");
   __syncthreads();
   // the C column and the Kutta row scaled by sf
-  for (int k = tid; k < m; k += kSmemLuThreads) {
+  for (int k = tid; k < m; k += NT) {
     F[n * ld + k] *= sf;
     if (k < n) F[k * ld + n] *= sf;
   }
   __syncthreads();
-  if (warp == 0) smem_diag_lu(F, ld, 0, min(NB, m), ipiv, bperm, red, cand);
+  auto diag = [&](int k, int kb) {
+    float* P = F + k * ld + k;
+    diag_lu([&](int r, int t) -> float& { return P[r * ld + t]; }, kb, ipiv + k, k, dt);
+  };
+  if (warp == 0) diag(0, min(NB, m));
   __syncthreads();
 
   for (int k0 = 0;; k0 += NB) {
-    if (cand[0] != 0ull) {
+    if (dt.fz != 0) {
       if (tid == 0) {
-        a.info[b] = k0 + (int)cand[0];
+        a.info[b] = k0 + dt.fz;
         if (a.iters) a.iters[b] = 0;
       }
       return;
     }
     const int kb = min(NB, m - k0);
     const int k1 = k0 + kb;
-    const float* P = F + k0 * ld + k0;
-    // ---- A: L21 = A21 U11^{-1} (also into LT), then the exchanges on the
-    // columns left of the panel (threads 0..255); U12 = L11^{-1} A12 with the
-    // rows read through the exchanges (threads 256..511) ----
-    if (tid < kSmemLuThreads / 2) {
-      const int r = k1 + tid;
-      if (r < m) {  // then kb == NB
-        float x[NB];
+    const int nw = (m - k1 + 31) >> 5;
+    // ---- A ---- (the warps of either half take 32 rows / columns each)
+    if (warp < NW / 2) {
+      for (int w = warp; w < nw + 1; w += NW / 2) {
+        float x[32];
+        if (w == 0) {
 #pragma unroll
-        for (int t = 0; t < NB; ++t) x[t] = F[r * ld + k0 + t];
-        // right-looking: once x_q is final it goes into every later column
-        // (the same terms in the same order as the row's dot products)
+          for (int t = 0; t < 32; ++t) x[t] = (t == lane) ? 1.0f : 0.0f;
+          float* G = F + (k0 + lane) * ld + k0;
+          tri_subst<true>(x, dt, [&](int q, float v) {
+            if (lane < kb && q < kb && q >= lane) G[q] = v;
+          });
+        } else {
+          const int r = k1 + 32 * (w - 1) + lane;
+          const bool ok = r < m;
+          float* G = F + (ok ? r : k0) * ld + k0;
+          float* T = LT + (r - k1);
 #pragma unroll
-        for (int q = 0; q < NB; ++q) {
-          x[q] *= (float)red[q];
-#pragma unroll
-          for (int t = q + 1; t < NB; ++t) x[t] = fmaf(-x[q], P[q * ld + t], x[t]);
-        }
-#pragma unroll
-        for (int t = 0; t < NB; ++t) {
-          F[r * ld + k0 + t] = x[t];
-          LT[t * ldt + tid] = x[t];
+          for (int t = 0; t < 32; ++t) x[t] = ok ? G[t] : 0.0f;
+          tri_subst<true>(x, dt, [&](int q, float v) {
+            if (ok) {
+              G[q] = v;
+              T[q * ldt] = v;
+            }
+          });
         }
       }
-      for (int c = tid; c < k0; c += kSmemLuThreads / 2) {
+    } else {
+      for (int w = warp - NW / 2; w < nw + 1; w += NW / 2) {
+        float x[32];
+        if (w == 0) {
+#pragma unroll
+          for (int t = 0; t < 32; ++t) x[t] = (t == lane) ? 1.0f : 0.0f;
+          float* G = F + k0 * ld + k0 + lane;
+          tri_subst<false>(x, dt, [&](int q, float v) {
+            if (q < kb && q > lane) G[q * ld] = v;
+          });
+        } else {
+          const int c = k1 + 32 * (w - 1) + lane;
+          const bool ok = c < m;
+          float* G = F + k0 * ld + (ok ? c : k0);
+#pragma unroll
+          for (int t = 0; t < 32; ++t) x[t] = ok ? G[dt.bperm[t] * ld] : 0.0f;
+          tri_subst<false>(x, dt, [&](int q, float v) {
+            if (ok) G[q * ld] = v;
+          });
+        }
+      }
+    }
+    // the exchanges on the columns left of the panel
+    if (dt.moved)
+      for (int c = tid; c < k0; c += NT) {
         float v[NB];
 #pragma unroll
-        for (int q = 0; q < NB; ++q) v[q] = (q < kb) ? F[(k0 + bperm[q]) * ld + c] : 0.0f;
+        for (int q = 0; q < NB; ++q) v[q] = (q < kb) ? F[(k0 + dt.bperm[q]) * ld + c] : 0.0f;
 #pragma unroll
         for (int q = 0; q < NB; ++q)
           if (q < kb) F[(k0 + q) * ld + c] = v[q];
       }
-    } else {
-      const int c = k1 + tid - kSmemLuThreads / 2;
-      if (c < m) {  // then kb == NB
-        float col[NB];
-#pragma unroll
-        for (int t = 0; t < NB; ++t) col[t] = F[(k0 + bperm[t]) * ld + c];
-#pragma unroll
-        for (int q = 0; q < NB; ++q) {
-          const float x = col[q];
-          F[(k0 + q) * ld + c] = x;
-#pragma unroll
-          for (int t = q + 1; t < NB; ++t) col[t] = fmaf(-P[t * ld + q], x, col[t]);
-        }
-      }
-    }
     __syncthreads();
     if (k1 >= m) break;
     const int kb2 = min(NB, m - k1);
     // ---- B: the next panel's columns [k1, k1 + kb2) ----
-    smem_update(F, ld, LT, ldt, m, k0, k1, kb, k1, k1 + kb2, 0, 32);
+    smem_update(F, ld, LT, ldt, m, k0, k1, k1, k1 + kb2, warp, NW, 32);
     __syncthreads();
     // ---- C: the next diagonal block (warp 0) | the remaining columns ----
+    // (warp 0 has its scheduler to itself: every fourth warp stays out)
     if (warp == 0)
-      smem_diag_lu(F, ld, k1, kb2, ipiv, bperm, red, cand);
-    else
-      smem_update(F, ld, LT, ldt, m, k0, k1, kb, k1 + kb2, m, 1, 128);
+      diag(k1, kb2);
+    else if (warp & 3)
+      smem_update(F, ld, LT, ldt, m, k0, k1, k1 + kb2, m, warp - 1 - (warp >> 2), 3 * NW / 4, 128);
     __syncthreads();
   }
-  // the 32 x 32 diagonal blocks inverted in place, a warp per triangle
-  {
-    const int nb = (m + NB - 1) / NB;
-    for (int t = warp; t < 2 * nb; t += kSmemLuWarps) {
-      const int d0 = NB * (t >> 1), kbd = min(NB, m - d0);
-      if (t & 1)
-        invert_upper(F + d0 * ld + d0, ld, kbd);
-      else
-        invert_lower_unit(F + d0 * ld + d0, ld, kbd);
-    }
-  }
-  __syncthreads();
   float* G = a.LU + moff;
-  for (int rr = warp; rr < m; rr += kSmemLuWarps)
+  for (int rr = warp; rr < m; rr += NW)
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
       const int cc = lane + 32 * u;
       if (cc < m) G[rr * m + cc] = F[rr * ld + cc];
     }
   int32_t* gpiv = a.piv + vec_off(bt, b);
-  for (int k = tid; k < m; k += kSmemLuThreads) gpiv[k] = ipiv[k];
+  for (int k = tid; k < m; k += NT) gpiv[k] = ipiv[k];
+}
+static_assert(kSmemLuM <= 256, "k_lu_smem writes rows of at most 8 x 32 columns");
+
+static size_t lu_smem_smem(int n_max) {
+  const size_t mv = (size_t)n_max + 1, ldv = mv | 1;
+  return sizeof(DiagTab) + 32 * 8 + 32 * (size_t)lu_smem_ldt((int)mv) * 4 + mv * 4 + mv * ldv * 4;
 }
 
-size_t lu_smem_smem(int n_max) {
-  const size_t mv = (size_t)n_max + 1, ldv = mv | 1, ldt = (mv + 7) & ~(size_t)7;
-  const size_t bytes = (mv * ldv * 4 + 15) & ~(size_t)15;
-  return bytes + 32 * ldt * 4 + 32 * 8 + 16 + mv * 4 + 32 * 4;
-}
-
-template <int NB>
-size_t lu_global_smem(int n_max) {
+static size_t lu_global_smem(int n_max) {
   const size_t mv = (size_t)n_max + 1;
-  size_t bytes = mv * (NB + 1) * 4 + (size_t)NB * 128 * 4;
-  bytes = (bytes + 15) & ~(size_t)15;
-  return bytes + 32 * 8 + kWarps * 8 + mv * 4 + NB * 4;
+  return sizeof(DiagTab) + 32 * (size_t)kSlabW * 4 + 32 * 8 +
+         32 * (size_t)lu_panel_ld((int)mv) * 4 + mv * 4;
 }
 
 // ---------------------------------------------------------------------------
@@ -1604,16 +1661,32 @@ static SolveArgs make_args(const Batch& bt, const float* A_hi, const float* A_lo
   return a;
 }
 
+// Which one-block LU a launch of B airfoils of at most mv unknowns takes (1 through
+// L2, 2 in shared memory).  Up to 128 unknowns several airfoils of the
+// shared-memory form fit an SM and it is the faster one at any batch (4096 of 100
+// panels: 531 us against 727; one: 45 / 62).  Above, one airfoil fills the SM's
+// shared memory: it wins by its shorter steps until three L2-resident airfoils
+// per SM hide each other's (160 panels: 1 airfoil 70 / 116 us, 304 138 / 138, 1216
+// 552 / 523; 200 panels: 1 93 / 161, 304 185 / 218, 1216 745 / 789, 4096 2478 /
+// 2321).  A launch that also holds larger airfoils runs them all through L2 at
+// once.
+static int lu_kind_by_size(int B, int mv) {
+  if (mv > kSmemLuM) return 1;
+  if (mv <= 128) return 2;
+  return B <= (mv <= 180 ? 2 : 12) * sm_count() ? 2 : 1;
+}
+
 // Factor every airfoil: with `inverse` the Gauss-Jordan inverse for m <= kGjM;
 // otherwise the one-block LU with the whole matrix in shared memory for m <=
-// kSmemLuM (lu_kind 0 or 2) or in the LU buffer through L2 (lu_kind 1, and
-// every m up to kLargeM); the step-synchronous blocked LU beyond.
+// kSmemLuM (lu_kind 2, or 0 and lu_kind_by_size) or in the LU buffer through L2
+// (lu_kind 1, and every m up to kLargeM); the step-synchronous blocked LU beyond.
 cudaError_t launch_lu_mixed(const Batch& bt, const float* A_hi, float* LU, int32_t* piv,
                             int32_t* info, int32_t* iters, bool inverse, cudaStream_t s,
                             int lu_kind) {
   SolveArgs a = make_args(bt, A_hi, nullptr, LU, piv, nullptr, nullptr, nullptr, nullptr,
                           nullptr, 0, 0.0, info, iters);
   a.inverse = inverse ? 1 : 0;
+  if (lu_kind == 0) lu_kind = lu_kind_by_size(bt.B, bt.n_max + 1);
   a.lu_kind = lu_kind;
   cudaError_t e;
   if (bt.n_max + 1 > kLargeM) {
@@ -1625,19 +1698,24 @@ cudaError_t launch_lu_mixed(const Batch& bt, const float* A_hi, float* LU, int32
     SolveArgs h = a;
     h.bt.n_max = min(bt.n_max, kSmemLuM - 1);
     const size_t hs = lu_smem_smem(h.bt.n_max);
-    e = ensure_smem(k_lu_smem, hs);
-    if (e != cudaSuccess) return e;
-    k_lu_smem<<<bt.B, kSmemLuThreads, hs, s>>>(h);
-    e = cudaGetLastError();
+    const int mv = h.bt.n_max + 1;
+    auto go = [&](auto kernel, int nt) {
+      const cudaError_t r = ensure_smem(kernel, hs);
+      if (r != cudaSuccess) return r;
+      kernel<<<bt.B, nt, hs, s>>>(h);
+      return cudaGetLastError();
+    };
+    e = mv <= 64 ? go(k_lu_smem<128, 5>, 128)
+                 : mv <= 128 ? go(k_lu_smem<256, 3>, 256) : go(k_lu_smem<512, 1>, 512);
     if (e != cudaSuccess) return e;
   }
   if ((bt.n_max + 1 > kSmemLuM || lu_kind == 1) && (bt.n_max + 1 > kGjM || !inverse)) {
     SolveArgs g = a;
     g.bt.n_max = min(bt.n_max, kLargeM - 1);
-    const size_t smem = lu_global_smem<32>(g.bt.n_max);
-    e = ensure_smem(k_lu_global<32>, smem);
+    const size_t smem = lu_global_smem(g.bt.n_max);
+    e = ensure_smem(k_lu_global, smem);
     if (e != cudaSuccess) return e;
-    k_lu_global<32><<<bt.B, kThreads, smem, s>>>(g);
+    k_lu_global<<<bt.B, kThreads, smem, s>>>(g);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }

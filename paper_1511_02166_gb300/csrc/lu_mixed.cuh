@@ -9,7 +9,7 @@ namespace panel {
 constexpr int kSmemM = 230;  // largest m = n + 1 of a Gauss-Jordan inverse in shared memory
 constexpr int kGjM = 288;    // m up to this: Gauss-Jordan inverse (k_gj_mixed.cu)
 constexpr int kLargeM = 640; // m above this takes the step-synchronous blocked factor
-constexpr int kSmemLuM = 224; // m up to this: LU with the whole matrix in shared memory
+constexpr int kSmemLuM = 222; // m up to this: LU with the whole matrix in shared memory
 constexpr int kNB = 32;      // panel width
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
@@ -33,7 +33,7 @@ struct SolveArgs {
   int n_cap;         // the caller's n_max (bt.n_max may be lowered to size a kernel)
   int rhs_kind;      // forward right-hand side: 0 rhs, 1 v m_y, 2 -v m_x (polar basis)
   int ir_shape;      // refinement block shape: 0 by size, 1..4 = 128x8, 256x4, 512x2, 1024x1
-  int lu_kind;       // LU of m <= kSmemLuM: 0/2 whole matrix in shared memory, 1 through L2
+  int lu_kind;       // LU of m <= kSmemLuM: 2 whole matrix in shared memory, 1 through L2
   // Transposed right-hand side of a vector-Jacobian product (vjp != 0):
   // w_cl[b] dCl/du + w_u + w_cp dCp/du (each may be NULL = 0), with the
   // strengths u_in of the forward solution; vjp == 0 is dCl/du alone.

@@ -81,7 +81,15 @@ def size_buckets(sorted_sizes, width, min_count=1):
 
 MODES = {"fp64": bd.PANEL_FP64, "mixed": bd.PANEL_MIXED}
 GJ_MAX_M = 288  # largest m = n + 1 that the library factors by Gauss-Jordan
-LU_SMEM_MAX_M = 224  # largest m whose LU the library can run in shared memory
+LU_SMEM_MAX_M = 222  # largest m whose LU the library can run in shared memory
+
+
+def lu_kind_by_size(count, m, sms):
+    """The one-block LU that the library takes by default for `count` airfoils of
+    at most m unknowns on `sms` multiprocessors (1 through L2, 2 in shared memory)."""
+    if m > LU_SMEM_MAX_M:
+        return 1
+    return 2 if m <= 128 or count <= (2 if m <= 180 else 12) * sms else 1
 
 
 def _require_cuda(device):
@@ -338,7 +346,8 @@ class PanelBatch:
                 if self.inverse[k]:
                     n += 1 + (m > 230) + (m > GJ_MAX_M)
                 else:
-                    n += (self.lu_kind[k] != 1) + (m > LU_SMEM_MAX_M or self.lu_kind[k] == 1)
+                    kind = self.lu_kind[k] or lu_kind_by_size(cnt, m, sms)
+                    n += (kind != 1) + (m > LU_SMEM_MAX_M or kind == 1)
                 if m > 640:
                     blocks = -(-m // 128)
                     n += 3 + blocks + 2 * (blocks - 1)
@@ -372,7 +381,7 @@ class PanelBatch:
           2. per bucket, the assembly (PANEL_TUNE_ROUNDS 0..6: near-field rounds, or
              both entries of a pair at once);
           3. per bucket, the solve (factor + refinement of both systems): the LU
-             (for m <= 224 with the matrix in shared memory or through L2,
+             (for m <= 222 with the matrix in shared memory or through L2,
              PANEL_TUNE_LU 2 / 1) or the Gauss-Jordan inverse (m <= 288), each
              with each refinement block shape (PANEL_TUNE_IR 0..5).
         Choices are cached by device, size bound and batch class

@@ -36,3 +36,22 @@ def test_split_adjoint_of_a_small_batch_matches_the_per_airfoil_kernel(sizes):
     for b in range(len(sizes)):
         a, c = (g[small.offsets[b]:small.offsets[b + 1]] for g in grads)
         assert np.max(np.abs(a - c)) <= 1e-11 * np.max(np.abs(c))
+
+
+@pytest.mark.parametrize("n", [3, 30, 31, 32, 62, 63, 64, 95, 126, 127, 128, 159, 191, 220, 221])
+def test_lu_in_shared_memory_and_through_l2_agree(n):
+    """Both one-block LUs do the same operations in the same order at every edge of
+    their 32-column panels and of the shared-memory form's block sizes."""
+    need_gpu()
+    from paper_1511_02166_gb300.solver import PanelBatch
+    pop = _airfoils((n, n, max(3, n - 1)), seed=n)
+    out = []
+    for kind in (1, 2):
+        pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, bucket_width=None)
+        pb.lu_kind = [kind]
+        pb.assemble()
+        pb.solve(stage="factor")
+        assert int(pb.info.abs().max()) == 0
+        out.append((pb.LU.cpu().numpy().view(np.uint32), pb.piv.cpu().numpy()))
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1], out[1][1])
