@@ -84,6 +84,16 @@ GJ_MAX_M = 288  # largest m = n + 1 that the library factors by Gauss-Jordan
 LU_SMEM_MAX_M = 222  # largest m whose LU the library can run in shared memory
 
 
+def assembly_spread(count, n_max, rounds, sms):
+    """Whether the library assembles `count` airfoils of at most n_max panels with
+    several blocks per airfoil (a preparing launch, then the pairs)."""
+    if rounds or n_max <= 64:
+        return rounds == 6
+    nch = -(-n_max // 64)
+    return count * nch * (nch + 1) // 2 <= sms or not (
+        n_max <= 128 or (n_max <= 224 and count > sms))
+
+
 def lu_kind_by_size(count, m, sms):
     """The one-block LU that the library takes by default for `count` airfoils of
     at most m unknowns on `sms` multiprocessors (1 through L2, 2 in shared memory)."""
@@ -328,8 +338,9 @@ class PanelBatch:
             self.run(with_grad=with_grad)
 
     def launches_per_step(self, with_grad: bool = True) -> int:
-        """Kernel launches of one step: per bucket assemble, factor, refine and
-        adjoint, plus one forces launch.  The mixed factor launches one kernel
+        """Kernel launches of one step: per bucket assemble (two when the pairs are
+        spread over several blocks per airfoil), factor, refine and adjoint, plus
+        one forces launch.  The mixed factor launches one kernel
         per size class the bucket may hold (Gauss-Jordan in shared memory and in
         global memory, or the one-block LU in shared memory and through L2) and,
         for m > 640 with T 128-column blocks, the step-synchronous LU: the tiled
@@ -341,7 +352,8 @@ class PanelBatch:
         sms = torch.cuda.get_device_properties(self.device).multi_processor_count
         for k, (start, cnt, nmax) in enumerate(self.buckets):
             m = nmax + 1
-            n += 1  # assemble
+            n += 1 + (self.flags == bd.PANEL_MIXED and
+                      assembly_spread(cnt, nmax, self.rounds[k], sms))
             if self.flags == bd.PANEL_MIXED:
                 if self.inverse[k]:
                     n += 1 + (m > 230) + (m > GJ_MAX_M)

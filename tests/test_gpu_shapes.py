@@ -55,3 +55,49 @@ def test_lu_in_shared_memory_and_through_l2_agree(n):
         out.append((pb.LU.cpu().numpy().view(np.uint32), pb.piv.cpu().numpy()))
     assert np.array_equal(out[0][0], out[1][0])
     assert np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("sizes", [(3, 70), (65, 96, 97), (127, 128, 129), (160,), (255, 257, 31),
+                                   (15, 16, 17, 400), (1030, 640)])
+@pytest.mark.parametrize("copies", [1, 40])
+def test_assembly_kernels_give_the_same_matrix(sizes, copies):
+    """The forms chosen by batch and size (split rows, tiles of 64 and 128 panels)
+    against one block per airfoil: every entry by the same operations."""
+    need_gpu()
+    from paper_1511_02166_gb300.solver import PanelBatch
+    base = _airfoils(sizes, seed=sum(sizes))
+    pop = inputs.pack([base.airfoil(b) for b in range(len(sizes))] * copies,
+                      np.tile(base.alpha, copies))
+    out = []
+    for rounds in (1, 0, 6):
+        pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, bucket_width=None)
+        for t in (pb.A_hi, pb.A_lo, pb.rhs):
+            t.fill_(float("nan"))
+        pb.rounds = [rounds]
+        pb.assemble()
+        assert int(pb.info.abs().max()) == 0
+        out.append([t.cpu().numpy() for t in (pb.A_hi, pb.A_lo, pb.rhs)])
+        assert all(np.isfinite(t).all() for t in out[-1])
+    for other in out[1:]:
+        assert np.array_equal(out[0][0].view(np.uint32), other[0].view(np.uint32))
+        assert np.array_equal(out[0][1].view(np.uint32), other[1].view(np.uint32))
+        assert np.max(np.abs(out[0][2] - other[2])) <= 1e-15
+
+
+@pytest.mark.parametrize("n", [80, 300])
+def test_assembly_of_a_small_batch_reports_bad_geometry(n):
+    """The codes of the several-block forms: clockwise, zero panel, non-finite, good."""
+    need_gpu()
+    import torch
+    from paper_1511_02166_gb300.solver import PanelBatch
+    good = inputs.naca4(0.02, 0.4, 0.12, n)
+    zero, nan = good.copy(), good.copy()
+    zero[n - 1] = zero[0]
+    nan[n // 2, 1] = np.nan
+    pop = inputs.pack([good[::-1].copy(), zero, nan, good], [0.05] * 4)
+    pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, bucket_width=None)
+    pb.run(with_grad=True)
+    torch.cuda.synchronize()
+    assert pb.info.cpu().tolist() == [-2, -3, -4, 0]
+    assert torch.isnan(pb.cl[:3]).all() and torch.isfinite(pb.cl[3])
+    assert torch.isfinite(pb.grad[-n:]).all() and torch.isnan(pb.grad[:-n]).all()
