@@ -1202,18 +1202,116 @@ __device__ __forceinline__ double resacc_sub_from(double c, const LiteAcc& a) {
   return c - ((double)a.s.hi + (double)a.s.lo);
 }
 
+__device__ __forceinline__ ResAcc shfl_xor_acc(const ResAcc& a, int o) {
+  ResAcc b;
+  b.s1 = __shfl_xor_sync(0xffffffffu, a.s1, o);
+  b.s2.hi = __shfl_xor_sync(0xffffffffu, a.s2.hi, o);
+  b.s2.lo = __shfl_xor_sync(0xffffffffu, a.s2.lo, o);
+  b.s3 = __shfl_xor_sync(0xffffffffu, a.s3, o);
+  return b;
+}
+__device__ __forceinline__ LiteAcc shfl_xor_acc(const LiteAcc& a, int o) {
+  LiteAcc b;
+  b.s.hi = __shfl_xor_sync(0xffffffffu, a.s.hi, o);
+  b.s.lo = __shfl_xor_sync(0xffffffffu, a.s.lo, o);
+  return b;
+}
+__device__ __forceinline__ ResAcc sel_acc(bool c, const ResAcc& a, const ResAcc& b) {
+  ResAcc r;
+  r.s1 = c ? a.s1 : b.s1;
+  r.s2.hi = c ? a.s2.hi : b.s2.hi;
+  r.s2.lo = c ? a.s2.lo : b.s2.lo;
+  r.s3 = c ? a.s3 : b.s3;
+  return r;
+}
+__device__ __forceinline__ LiteAcc sel_acc(bool c, const LiteAcc& a, const LiteAcc& b) {
+  LiteAcc r;
+  r.s.hi = c ? a.s.hi : b.s.hi;
+  r.s.lo = c ? a.s.lo : b.s.lo;
+  return r;
+}
+
+// Residuals of a warp's rows j = first + step i (i = 0, 1, ...), four at a time:
+// add() takes the lanes' shares of one row after the other.  Two halving exchanges
+// (each lane keeps half of the rows) and three butterflies sum four rows over the
+// lanes with 6 merges instead of 20, and the FP64 part (the right-hand side, the
+// final subtraction) waits until every lane has a row of its own: on a pipe of 1/74
+// of the FP32 rate it was one lane's chain of dependent operations per row.  QUAD
+// false sums each row by itself (the fused pass has no registers for four).
+template <class Acc, class Rhs, class RT, bool QUAD = true>
+struct RowSums {
+  Acc v[4], keep;
+  int i = 0;  // rows taken
+  const Rhs& b;
+  RT* r;
+  int first, step, m;
+  __device__ RowSums(const Rhs& b_, RT* r_, int first_, int step_, int m_)
+      : b(b_), r(r_), first(first_), step(step_), m(m_) {
+#pragma unroll
+    for (int t = 0; t < 4; ++t) resacc_init(v[t]);
+    resacc_init(keep);
+  }
+  __device__ __forceinline__ void add(const Acc& a) {
+    if constexpr (!QUAD) {
+      keep = sel_acc((int)(threadIdx.x & 31) == (i & 31), warp_sum_res(a), keep);
+      if ((++i & 31) == 0) flush(i - 32);
+      return;
+    }
+    v[0] = v[1];
+    v[1] = v[2];
+    v[2] = v[3];
+    v[3] = a;
+    if ((++i & 3) == 0) reduce();
+  }
+  __device__ __forceinline__ void reduce() {
+    const int lane = threadIdx.x & 31;
+    const bool b4 = (lane & 16) != 0, b3 = (lane & 8) != 0;
+    Acc k0 = sel_acc(b4, v[2], v[0]), k1 = sel_acc(b4, v[3], v[1]);
+    resacc_merge(k0, shfl_xor_acc(sel_acc(b4, v[0], v[2]), 16));
+    resacc_merge(k1, shfl_xor_acc(sel_acc(b4, v[1], v[3]), 16));
+    Acc k = sel_acc(b3, k1, k0);
+    resacc_merge(k, shfl_xor_acc(sel_acc(b3, k0, k1), 8));
+#pragma unroll 1
+    for (int o = 4; o > 0; o >>= 1) resacc_merge(k, shfl_xor_acc(k, o));
+    // the lanes l >> 3 == t hold row t of the four; lane l keeps the group l & 7
+    keep = sel_acc((lane & 7) == ((i >> 2) - 1 & 7), k, keep);
+    if ((i & 31) == 0) flush(i - 32);
+  }
+  __device__ __forceinline__ void flush(int i0) {
+    const int lane = threadIdx.x & 31;
+    const int row = i0 + (QUAD ? 4 * (lane & 7) + (lane >> 3) : lane);
+    const int j = first + step * row;
+    if (row < i && j < m) b.store(r, j, resacc_sub_from(b(j), keep));
+  }
+  __device__ __forceinline__ void finish() {
+    const int n = i;
+    if constexpr (QUAD) {
+      Acc z;
+      resacc_init(z);
+      while (i & 3) add(z);
+    }
+    if (i & 31) {
+      const int i0 = i & ~31;
+      i = n;
+      flush(i0);
+    }
+  }
+};
+
 // r_j = b_j - sum_i M_ji x_i for all rows j; x given as float pairs (xh, xl).
-// A warp takes two rows at a time and issues all loads of a 256-column chunk
-// before accumulating.
+// A warp takes two neighbouring rows at a time and issues all loads of a
+// 256-column chunk before accumulating.
 template <class Acc, class Rhs, class RT>
 __device__ void residual_rows(const float* __restrict__ Ah, const float* __restrict__ Al, int m,
                               const float* xh, const float* xl, const Rhs& b, RT* r) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int j0 = 2 * warp; j0 < m; j0 += 2 * (int)(blockDim.x >> 5)) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  RowSums<Acc, Rhs, RT> sums(b, r, warp, nw, m);
+  for (int j0 = warp; j0 < m; j0 += 2 * nw) {
     Acc acc0, acc1;
     resacc_init(acc0);
     resacc_init(acc1);
-    const bool two = j0 + 1 < m;
+    const int j1 = j0 + nw;
+    const bool two = j1 < m;
     for (int c0 = 0; c0 < m; c0 += 256) {
       float h0[8], l0[8], h1[8], l1[8];
 #pragma unroll
@@ -1222,8 +1320,8 @@ __device__ void residual_rows(const float* __restrict__ Ah, const float* __restr
         const bool ok = c < m;
         h0[t] = ok ? __ldg(Ah + j0 * m + c) : 0.0f;
         l0[t] = ok ? __ldg(Al + j0 * m + c) : 0.0f;
-        h1[t] = (ok && two) ? __ldg(Ah + (j0 + 1) * m + c) : 0.0f;
-        l1[t] = (ok && two) ? __ldg(Al + (j0 + 1) * m + c) : 0.0f;
+        h1[t] = (ok && two) ? __ldg(Ah + j1 * m + c) : 0.0f;
+        l1[t] = (ok && two) ? __ldg(Al + j1 * m + c) : 0.0f;
       }
 #pragma unroll
       for (int t = 0; t < 8; ++t) {
@@ -1235,13 +1333,10 @@ __device__ void residual_rows(const float* __restrict__ Ah, const float* __restr
         }
       }
     }
-    acc0 = warp_sum_res(acc0);
-    acc1 = warp_sum_res(acc1);
-    if (lane == 0) {
-      b.store(r, j0, resacc_sub_from(b(j0), acc0));
-      if (two) b.store(r, j0 + 1, resacc_sub_from(b(j0 + 1), acc1));
-    }
+    sums.add(acc0);
+    sums.add(acc1);
   }
+  sums.finish();
 }
 
 // r_i = g_i - sum_j M_ji x_j for all columns i: each warp owns 32 consecutive
@@ -1287,6 +1382,7 @@ __device__ void residual_both(const float* __restrict__ Ah, const float* __restr
   Acc cacc[FT];
 #pragma unroll
   for (int t = 0; t < FT; ++t) resacc_init(cacc[t]);
+  RowSums<Acc, Rhs, RT, false> sums(b, rf, warp, (int)(blockDim.x >> 5), m);
   for (int j = warp; j < m; j += (int)(blockDim.x >> 5)) {
     float h[FT], l[FT];
 #pragma unroll
@@ -1307,9 +1403,9 @@ __device__ void residual_both(const float* __restrict__ Ah, const float* __restr
         resacc_add(cacc[t], h[t], l[t], yjh, yjl);
       }
     }
-    racc = warp_sum_res(racc);
-    if (lane == 0) b.store(rf, j, resacc_sub_from(b(j), racc));
+    sums.add(racc);
   }
+  sums.finish();
 #pragma unroll
   for (int t = 0; t < FT; ++t) {
     const int c = lane + 32 * t;
@@ -1359,6 +1455,22 @@ struct IrRhs {
   double w_cl;
   int n, q, rhs_kind, vjp;
   double v, cc, s;
+  __device__ void init(const SolveArgs& a, int b, int n_, int q_, double s_) {
+    const int64_t vo = vec_off(a.bt, b);
+    rhs = (a.rhs_kind == 0 && a.rhs) ? a.rhs + vo : nullptr;
+    nd = a.bt.nodes + 2 * a.bt.node_off[b];
+    w_u = a.w_u ? a.w_u + vo : nullptr;
+    w_cp = a.w_cp ? a.w_cp + a.bt.node_off[b] : nullptr;
+    u_in = a.u_in ? a.u_in + vo : nullptr;
+    w_cl = a.w_cl ? a.w_cl[b] : 0.0;
+    n = n_;
+    q = q_;
+    rhs_kind = a.rhs_kind;
+    vjp = a.vjp;
+    v = a.vinf ? a.vinf[b] : 1.0;
+    cc = a.chord ? a.chord[b] : 1.0;
+    s = s_;
+  }
   __device__ double operator()(int k) const { return eval(k); }
   __device__ double eval(int k) const {
     if (q == 0) {
@@ -1396,6 +1508,33 @@ __device__ __forceinline__ float solve_input(float r, int, int, double) { return
 
 __device__ __forceinline__ int gpiv_first(const SolveArgs& a, int b) {
   return a.piv[vec_off(a.bt, b)];
+}
+
+// Row permutation of the factor, P y = y[perm], from its exchanges (by the whole
+// block; ends with a barrier).  Every exchange stays inside its diagonal block
+// (32 rows, or the blocks of the tiled layout), so the blocks' exchanges are
+// composed side by side, a thread each, instead of one thread walking all m
+// (~45 cycles a row: 20 k of a 200-panel airfoil's 600 k cycles).
+__device__ __forceinline__ void factor_permutation(const int32_t* gpiv, int m, bool gj, int* perm) {
+  for (int k = threadIdx.x; k < m; k += blockDim.x) perm[k] = k;
+  __syncthreads();
+  const bool tiled = !gj && m > kLargeM;
+  const int blk = tiled ? kTlB : 32;
+  const int e = tiled ? m - kTlB * ((m - 1) / kTlB) : 32;  // size of the first block
+  const int k0 = threadIdx.x == 0 ? 0 : e + blk * ((int)threadIdx.x - 1);
+  if (k0 < m) {
+    const int k1 = min(m, threadIdx.x == 0 ? e : k0 + blk);
+#pragma unroll 8
+    for (int k = k0; k < k1; ++k) {
+      const int p = gj ? -gpiv[k] - 1 : gpiv[k];
+      if (p != k) {
+        const int t = perm[k];
+        perm[k] = perm[p];
+        perm[p] = t;
+      }
+    }
+  }
+  __syncthreads();
 }
 
 // NT threads, MINB blocks per SM (see launch_ir_kernel).
@@ -1467,22 +1606,7 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
 
   // right-hand sides: b, and g = dCl/du = 2 |h_k| / (v c) (0 for C); x = 0, r = b
   IrRhs rhs[2];
-  for (int q = 0; q < 2; ++q) {
-    const int64_t vo = vec_off(bt, b);
-    rhs[q].rhs = (a.rhs_kind == 0 && a.rhs) ? a.rhs + vo : nullptr;
-    rhs[q].nd = bt.nodes + 2 * bt.node_off[b];
-    rhs[q].w_u = a.w_u ? a.w_u + vo : nullptr;
-    rhs[q].w_cp = a.w_cp ? a.w_cp + bt.node_off[b] : nullptr;
-    rhs[q].u_in = a.u_in ? a.u_in + vo : nullptr;
-    rhs[q].w_cl = a.w_cl ? a.w_cl[b] : 0.0;
-    rhs[q].n = n;
-    rhs[q].q = q;
-    rhs[q].rhs_kind = a.rhs_kind;
-    rhs[q].vjp = a.vjp;
-    rhs[q].v = a.vinf ? a.vinf[b] : 1.0;
-    rhs[q].cc = a.chord ? a.chord[b] : 1.0;
-    rhs[q].s = s;
-  }
+  for (int q = 0; q < 2; ++q) rhs[q].init(a, b, n, q, s);
   SmemRhs srhs[2];
   srhs[0].bb = bbs;
   srhs[1].bb = bbs + mv;
@@ -1503,21 +1627,12 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
       }
     }
   }
-  // row permutation of the factor: P y = y[perm]
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < m; ++k) perm[k] = k;
-    for (int k = 0; k < m; ++k) {
-      const int p = gj ? -gpiv[k] - 1 : gpiv[k];
-      const int t = perm[k];
-      perm[k] = perm[p];
-      perm[p] = t;
-    }
-  }
-  __syncthreads();
+  factor_permutation(gpiv, m, gj, perm);
 
   bool active[2] = {act0, act1};
   bool conv[2] = {!act0, !act1};
-  double dprev[2] = {0.0, 0.0};  // size of the previous correction
+  float dprev[2] = {0.0f, 0.0f};  // size of the previous correction
+  const float tol = (float)a.tol;
   int it = 0;
   for (;; ++it) {
     const bool run0 = active[0] && !conv[0], run1 = active[1] && !conv[1];
@@ -1546,26 +1661,24 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
       if (!(q == 0 ? run0 : run1)) continue;
       IrSystem<RT>& S = sys[q];
       const float* w = (q == 0) ? y : z;
-      double dmax = 0.0;
+      float dmax = 0.0f, xmax = 0.0f;
       for (int k = threadIdx.x; k < m; k += (int)blockDim.x) {
         const int dst = (q == 0) ? k : perm[k];
         const double d = (dst == n) ? (double)w[k] * s : (double)w[k];
-        S.x[dst] += d;
-        dmax = fmax(dmax, fabs(d));
+        const double xn = S.x[dst] + d;
+        S.x[dst] = xn;
+        dmax = fmaxf(dmax, fabsf((float)d));
+        xmax = fmaxf(xmax, fabsf((float)xn));
       }
-      __syncthreads();
-      double xmax = 0.0;
-      for (int k = threadIdx.x; k < m; k += (int)blockDim.x) xmax = fmax(xmax, fabs(S.x[k]));
-      dmax = block_absmax_d(dmax, red);
-      xmax = block_absmax_d(xmax, red);
+      block_max2(dmax, xmax, red);
       // Converged when the correction just applied is below tol |x|, or when
       // the contraction seen over the last two corrections (rho = |d_k| /
       // |d_{k-1}| <= 1/8) predicts the next one, |d_k| rho, below tol |x|: the
       // error left in x_{k+1} is about that next correction.
       // (the correction of iteration 1 comes from the double-float residual,
       // so the first test waits for iteration 2)
-      if (it >= 2 && dmax <= a.tol * xmax) conv[q] = true;
-      if (it >= 2 && dmax <= 0.125 * dprev[q] && dmax * (dmax / dprev[q]) <= a.tol * xmax)
+      if (it >= 2 && dmax <= tol * xmax) conv[q] = true;
+      if (it >= 2 && dmax <= 0.125f * dprev[q] && dmax * (dmax / dprev[q]) <= tol * xmax)
         conv[q] = true;
       dprev[q] = dmax;
     }
@@ -1631,6 +1744,10 @@ size_t ir_mixed_smem(int n_max, int nt) {
   const size_t vecs = (mv <= (size_t)kFuseM) ? 6 * mv * 8 + 5 * mv * 4 : 7 * mv * 4;
   return 32 * 8 + vecs + mv * 4 + 32 * 4 + 32 + part;
 }
+
+}  // namespace panel
+#include "ir_cluster.cuh"
+namespace panel {
 
 static SolveArgs make_args(const Batch& bt, const float* A_hi, const float* A_lo, float* LU,
                            int32_t* piv, const double* rhs, const double* vinf,
@@ -1748,11 +1865,69 @@ static cudaError_t launch_ir_shape(const SolveArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+static cudaLaunchConfig_t ir_cluster_config(int B, int n_max, int C, cudaStream_t s,
+                                            cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(B * C);
+  cfg.blockDim = dim3(kIrClThreads);
+  cfg.dynamicSmemBytes = ir_cluster_smem(n_max);
+  cfg.stream = s;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = C;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Clusters of C blocks of k_ir_cluster the device holds at once (asked once per
+// device, for the largest airfoil; 0 if the query fails).
+static int ir_cluster_capacity(int C) {
+  static std::mutex mu;
+  static std::map<std::pair<int, int>, int> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto it = known.find(std::make_pair(dev, C));
+  if (it != known.end()) return it->second;
+  int n = 0;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = ir_cluster_config(1, PANEL_N_MAX, C, nullptr, &at);
+  if (ensure_smem(k_ir_cluster, cfg.dynamicSmemBytes) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, k_ir_cluster, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    n = 0;
+  }
+  known[std::make_pair(dev, C)] = n;
+  return n;
+}
+
+// Blocks per airfoil of a refinement by clusters, or 0 for k_ir_mixed: the most that
+// let every airfoil of the batch run at once.  Measured, both systems (us, k_ir_mixed /
+// clusters of 1, 2, 4, 8): 1 airfoil of 100 panels 126 / 134, 128, 124, 126; of 160
+// 223 / 200, 182, 175, 173; of 600 1370 / 996, 711, 587, 544; of 1024 4284 / 3581,
+// 2444, 1589, 1337; of 2048 11315 / 13937, 8303, 5719, 3578; 76 airfoils of 300 569 /
+// 411, 338; of 1024 7083 / 4802, 3210; 18 of 2048 14263 / 15700, 9393, 6256.
+static int ir_cluster_blocks(const SolveArgs& a) {
+  const int mv = a.bt.n_max + 1;
+  if (a.ir_shape != 0 || mv <= 128) return 0;
+  for (int C = 8; C >= 1; C >>= 1)
+    if (a.bt.B <= ir_cluster_capacity(C)) return (C == 1 && mv > 1400) ? 0 : C;
+  return 0;
+}
+
+static cudaError_t launch_ir_cluster(const SolveArgs& a, int C, cudaStream_t s) {
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = ir_cluster_config(a.bt.B, a.bt.n_max, C, s, &at);
+  return cudaLaunchKernelEx(&cfg, k_ir_cluster, a);
+}
+
 static cudaError_t launch_ir_kernel(const SolveArgs& a, cudaStream_t s) {
   const int n_max = a.bt.n_max;
   auto fits = [&](int nt, int blocks) {
     return (size_t)blocks * (ir_mixed_smem(n_max, nt) + 1024) <= 233472;
   };
+  if (const int c = ir_cluster_blocks(a)) return launch_ir_cluster(a, c, s);
   // an explicit shape (autotuning), when one block of it fits the shared memory
   switch (a.ir_shape) {
     case 1:

@@ -44,17 +44,23 @@ struct SolveArgs {
   const double* u_in;  // [sum m_b]
 };
 
-__device__ __forceinline__ double block_absmax_d(double v, double* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = warp_max(v);
+// Block-wide maxima of two non-negative floats, in place (`red`: 64 words of shared
+// memory; all threads call it).  The sizes a stopping rule compares need no FP64: in
+// doubles, with every thread taking the maximum over the warps, they were 12 % of a
+// 100-panel refinement.
+__device__ __forceinline__ void block_max2(float& a, float& b, double* red) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  unsigned* w = reinterpret_cast<unsigned*>(red);
+  const unsigned ua = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
+  const unsigned ub = __reduce_max_sync(0xffffffffu, __float_as_uint(b));
   __syncthreads();
-  if (lane == 0) red[warp] = v;
+  if (lane == 0) {
+    w[warp] = ua;
+    w[32 + warp] = ub;
+  }
   __syncthreads();
-  double r = 0.0;
-  const int nw = blockDim.x >> 5;
-  for (int w = 0; w < nw; ++w) r = fmax(r, red[w]);
-  __syncthreads();
-  return r;
+  a = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < nw ? w[lane] : 0u));
+  b = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < nw ? w[32 + lane] : 0u));
 }
 
 // border scale s = mean |A_jj| over the influence block (hi plane)

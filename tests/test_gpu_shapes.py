@@ -101,3 +101,49 @@ def test_assembly_of_a_small_batch_reports_bad_geometry(n):
     assert pb.info.cpu().tolist() == [-2, -3, -4, 0]
     assert torch.isnan(pb.cl[:3]).all() and torch.isfinite(pb.cl[3])
     assert torch.isfinite(pb.grad[-n:]).all() and torch.isnan(pb.grad[:-n]).all()
+
+
+@pytest.mark.parametrize("sizes", [(128,), (129, 200, 160), (287, 288), (300, 639, 640), (641, 767),
+                                   (1024, 1040, 700, 40)])
+@pytest.mark.parametrize("copies", [1, 12, 30])
+def test_cluster_refinement_matches_the_one_block_refinement(sizes, copies):
+    """A batch that fits the chip as clusters of 8, 4, 2 or 1 blocks against the
+    explicit one-block shape: both end within the tolerance of the same solution
+    (up to 700 panels far below it; the larger airfoils' conditioning is 1e9)."""
+    need_gpu()
+    import torch
+    from paper_1511_02166_gb300.solver import PanelBatch
+    base = _airfoils(sizes, seed=len(sizes) + sizes[0])
+    pop = inputs.pack([base.airfoil(b) for b in range(len(sizes))] * copies,
+                      np.tile(base.alpha, copies))
+    out = []
+    for shape in (4, 0):
+        pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, bucket_width=None)
+        pb.ir_shape = [shape]
+        pb.run(with_grad=True)
+        cl = pb.polar(torch.tensor([[0.0, 0.1]] * pop.batch))
+        assert int(pb.info.abs().max()) == 0
+        out.append([t.cpu().numpy() for t in (pb.u, pb.lam, cl)])
+    for a, c in zip(out[0][:2], out[1][:2]):
+        for b in range(pop.batch):
+            o, n = pop.offsets[b] + b, pop.offsets[b + 1] - pop.offsets[b]
+            tol = 1e-11 if n <= 700 else 1e-10
+            assert np.max(np.abs(a[o:o + n + 1] - c[o:o + n + 1])) <= tol * np.max(np.abs(a[o:o + n + 1])), b
+    assert np.max(np.abs(out[0][2] - out[1][2])) <= 1e-11
+
+
+@pytest.mark.parametrize("n", [130, 260])
+def test_cluster_refinement_with_the_inverse(n):
+    """The Gauss-Jordan inverse through the cluster refinement."""
+    need_gpu()
+    from paper_1511_02166_gb300.solver import PanelBatch
+    pop = _airfoils((n, n - 1, 50), seed=n)
+    out = []
+    for inverse in (False, True):
+        pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, bucket_width=None)
+        pb.inverse = [inverse]
+        pb.run(with_grad=True)
+        assert int(pb.info.abs().max()) == 0
+        out.append((pb.u.cpu().numpy(), pb.grad.cpu().numpy()))
+    assert np.max(np.abs(out[0][0] - out[1][0])) <= 1e-11 * np.max(np.abs(out[0][0]))
+    assert np.max(np.abs(out[0][1] - out[1][1])) <= 1e-10 * np.max(np.abs(out[0][1]))
