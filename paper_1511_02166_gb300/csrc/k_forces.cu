@@ -11,26 +11,30 @@
 
 namespace panel {
 
-// One warp per airfoil.
-__global__ void __launch_bounds__(256) k_forces(Batch bt, const double* __restrict__ u,
-                                                const double* __restrict__ alpha,
-                                                const double* __restrict__ vinf,
-                                                const double* __restrict__ chord,
-                                                const int32_t* __restrict__ info,
-                                                double* __restrict__ cp, double* __restrict__ cl,
-                                                double* __restrict__ cl_p,
-                                                double* __restrict__ cd_p) {
-  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (w >= bt.B) return;
-  const int b = w;
+// The FP64 pipe is the bound (a square root and ~25 more operations per node, the sine
+// and cosine per airfoil), so what counts is how many SMs share the work.  WPA = 1: a
+// warp per airfoil, eight to a block, for full batches; WPA = 4: a block of four warps
+// per airfoil, so that a small batch reaches as many SMs as it has airfoils and a
+// large airfoil's nodes are walked by 128 lanes (64 of 100 panels: 22 -> 9 us, 24 of
+// 50..2047: 101 -> 26 us; 4096 of 200: 83 -> 70 us without the division by 1).
+template <int WPA>
+__global__ void __launch_bounds__(WPA == 1 ? 256 : 128) k_forces(
+    Batch bt, const double* __restrict__ u, const double* __restrict__ alpha,
+    const double* __restrict__ vinf, const double* __restrict__ chord,
+    const int32_t* __restrict__ info, double* __restrict__ cp, double* __restrict__ cl,
+    double* __restrict__ cl_p, double* __restrict__ cd_p) {
+  __shared__ double part[WPA == 1 ? 1 : 3 * WPA];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int b = WPA == 1 ? blockIdx.x * 8 + warp : blockIdx.x;
+  if (b >= bt.B) return;
   const int n = airfoil_n(bt, b);
   const double* x = bt.nodes + 2 * bt.node_off[b];
   const double* g = u + vec_off(bt, b);
   double* cpb = cp + bt.node_off[b];
+  const int t0 = WPA == 1 ? lane : threadIdx.x;
   if ((info && info[b] != 0) || n < 3) {
-    for (int j = lane; j < n; j += 32) cpb[j] = nan("");
-    if (lane == 0) {
+    for (int j = t0; j < n; j += 32 * WPA) cpb[j] = nan("");
+    if (t0 == 0) {
       cl[b] = nan("");
       if (cl_p) cl_p[b] = nan("");
       if (cd_p) cd_p[b] = nan("");
@@ -38,13 +42,15 @@ __global__ void __launch_bounds__(256) k_forces(Batch bt, const double* __restri
     return;
   }
   const double v = vinf ? vinf[b] : 1.0, c = chord ? chord[b] : 1.0;
+  double sa = 0.0, ca = 0.0;
+  if (warp % WPA == WPA - 1) sincos(alpha[b], &sa, &ca);
   double circ = 0.0, fx = 0.0, fy = 0.0;
-  for (int j = lane; j < n; j += 32) {
+  for (int j = t0; j < n; j += 32 * WPA) {
     const int j1 = (j + 1 == n) ? 0 : j + 1;
     const double hx = x[2 * j1] - x[2 * j], hy = x[2 * j1 + 1] - x[2 * j + 1];
     const double L = sqrt(hx * hx + hy * hy);
     const double gj = g[j];
-    const double q = gj / v;
+    const double q = vinf ? gj / v : gj;  // v is 1 without vinf
     const double cpj = 1.0 - q * q;
     cpb[j] = cpj;
     circ = fma(gj, L, circ);
@@ -54,20 +60,35 @@ __global__ void __launch_bounds__(256) k_forces(Batch bt, const double* __restri
   circ = warp_sum(circ);
   fx = warp_sum(fx);
   fy = warp_sum(fy);
+  if (WPA > 1) {
+    if (lane == 0) {
+      part[3 * warp] = circ;
+      part[3 * warp + 1] = fx;
+      part[3 * warp + 2] = fy;
+    }
+    __syncthreads();
+    if (warp != WPA - 1) return;
+    circ = fx = fy = 0.0;
+    for (int w = 0; w < WPA; ++w) {
+      circ += part[3 * w];
+      fx += part[3 * w + 1];
+      fy += part[3 * w + 2];
+    }
+  }
   if (lane == 0) {
-    const double a = alpha[b];
     cl[b] = 2.0 * circ / (v * c);
-    if (cl_p) cl_p[b] = (-fx * sin(a) + fy * cos(a)) / c;
-    if (cd_p) cd_p[b] = (fx * cos(a) + fy * sin(a)) / c;
+    if (cl_p) cl_p[b] = (-fx * sa + fy * ca) / c;
+    if (cd_p) cd_p[b] = (fx * ca + fy * sa) / c;
   }
 }
 
 cudaError_t launch_forces(const Batch& bt, const double* u, const double* alpha,
                           const double* vinf, const double* chord, const int32_t* info,
                           double* cp, double* cl, double* cl_p, double* cd_p, cudaStream_t s) {
-  const int wpb = 8;
-  const int grid = (bt.B + wpb - 1) / wpb;
-  k_forces<<<grid, wpb * 32, 0, s>>>(bt, u, alpha, vinf, chord, info, cp, cl, cl_p, cd_p);
+  if (bt.B <= 4 * sm_count())
+    k_forces<4><<<bt.B, 128, 0, s>>>(bt, u, alpha, vinf, chord, info, cp, cl, cl_p, cd_p);
+  else
+    k_forces<1><<<(bt.B + 7) / 8, 256, 0, s>>>(bt, u, alpha, vinf, chord, info, cp, cl, cl_p, cd_p);
   return cudaGetLastError();
 }
 
