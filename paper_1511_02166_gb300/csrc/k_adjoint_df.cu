@@ -588,6 +588,16 @@ size_t adjoint_df_smem(int n_max) {
          (size_t)kPanelFields * n_max * 4 + (size_t)8 * n_max * 16;
 }
 
+// The terms of the gradient that need no pair sums, into every node.
+cudaError_t launch_adjoint_prepare(const Batch& bt, const double* u, const double* lambda,
+                                   const double* alpha, const double* vinf, const double* chord,
+                                   const double* grad_cl, double* grad, const int32_t* info,
+                                   bool lam_weighted, cudaStream_t s) {
+  k_adjoint_prepare<<<dim3(bt.B, (bt.n_max + 255) / 256), 256, 0, s>>>(
+      bt, u, lambda, alpha, vinf, chord, grad_cl, grad, info, lam_weighted ? 1 : 0);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_adjoint_df(const Batch& bt, const double* u, const double* lambda,
                               const double* alpha, const double* vinf, const double* chord,
                               const double* grad_cl, double* grad, const int32_t* info,
@@ -604,9 +614,8 @@ cudaError_t launch_adjoint_df(const Batch& bt, const double* u, const double* la
     const size_t smem = adjoint_split_smem();
     e = ensure_smem(k_adjoint_df_split, smem);
     if (e != cudaSuccess) return e;
-    k_adjoint_prepare<<<dim3(bt.B, (bt.n_max + 255) / 256), 256, 0, s>>>(
-        bt, u, lambda, alpha, vinf, chord, grad_cl, grad, info, lam_weighted ? 1 : 0);
-    e = cudaGetLastError();
+    e = launch_adjoint_prepare(bt, u, lambda, alpha, vinf, chord, grad_cl, grad, info,
+                               lam_weighted, s);
     if (e != cudaSuccess) return e;
     const dim3 grid(bt.B, (bt.n_max + kSplitCols - 1) / kSplitCols, (bt.n_max + rows - 1) / rows);
     k_adjoint_df_split<<<grid, kSplitCols, smem, s>>>(bt, u, lambda, grad_cl, grad, info,

@@ -5,32 +5,35 @@
 // and b_j = v_inf (y_{j+1/2} cos a - x_{j+1/2} sin a).  The printed integral
 // uses two log and two atan2 per pair; here the two atan2 of one pair are
 // combined into one (their difference is the angle the panel subtends, always
-// inside (-pi, pi)), which leaves two log and one atan2 in native FP64.
+// inside (-pi, pi)), and the logarithms are those of the distances to the two
+// end nodes, which neighbouring panels share: one log and one atan2 per pair in
+// native FP64.  The FP64 pipe (16 G log/s, 12 G atan2/s on the whole chip) is
+// the bound; a block takes a range of rows, so that a batch of fewer airfoils
+// than SMs still uses every SM's pipe.
 #include "panel_common.cuh"
 
 namespace panel {
 
 // (1/2pi) * integral over the panel a->b of log|p - s| ds, in the panel frame
-// xi = (p-a).t, eta = (p-a).n (n = t rotated by +90 degrees), L = |b-a|:
-//   G = (1/2pi) [ xi/2 log r1^2 - (xi-L)/2 log r2^2 + eta*theta - L ],
+// xi = (p-a).t, eta = (p-a).n (n = t rotated by +90 degrees), L = |b-a|, with
+// la = log|p-a|^2 and lb = log|p-b|^2:
+//   G = (1/2pi) [ xi/2 la - (xi-L)/2 lb + eta*theta - L ],
 //   theta = atan2(eta L, xi (xi - L) + eta^2).
-__device__ __forceinline__ double panel_G_f64(double px, double py, double ax, double ay,
+__device__ __forceinline__ double panel_G_f64(double dx, double dy, double la, double lb,
                                               double tx, double ty, double L) {
-  double dx = px - ax, dy = py - ay;
   double xi = dx * tx + dy * ty;
   double eta = dy * tx - dx * ty;
   double xl = xi - L;
-  double r1 = xi * xi + eta * eta;
-  double r2 = xl * xl + eta * eta;
   double th = atan2(eta * L, xi * xl + eta * eta);
-  return kInvTwoPi * (0.5 * xi * log(r1) - 0.5 * xl * log(r2) + eta * th - L);
+  return kInvTwoPi * (0.5 * xi * la - 0.5 * xl * lb + eta * th - L);
 }
 
+// Block (x, y): the rows [rows y, rows y + rows) of airfoil order[x].
 __global__ void __launch_bounds__(256) k_assemble_f64(Batch bt, const double* __restrict__ alpha,
                                                       const double* __restrict__ vinf,
                                                       double* __restrict__ A,
                                                       double* __restrict__ rhs,
-                                                      int32_t* __restrict__ info) {
+                                                      int32_t* __restrict__ info, int rows) {
   extern __shared__ double sm[];
   const int b = bt.order[blockIdx.x];
   const int n = airfoil_n(bt, b);
@@ -45,12 +48,15 @@ __global__ void __launch_bounds__(256) k_assemble_f64(Batch bt, const double* __
   double* scratch = mys + bt.n_max;
 
   const double* nodes = bt.nodes + 2 * bt.node_off[b];
+  const bool first = blockIdx.y == 0 && threadIdx.x == 0;
   if (n > bt.n_max) {
-    if (threadIdx.x == 0) info[b] = PANEL_INFO_TOO_LARGE;
+    if (first) info[b] = PANEL_INFO_TOO_LARGE;
     return;
   }
+  const int j0 = blockIdx.y * rows;
+  if (j0 > n && blockIdx.y > 0) return;
   int st = load_and_check_geometry(nodes, n, xs, ys, scratch);
-  if (threadIdx.x == 0) info[b] = st;
+  if (first) info[b] = st;
   if (st != 0) return;
   for (int k = threadIdx.x; k < n; k += blockDim.x) {
     int k1 = (k + 1 == n) ? 0 : k + 1;
@@ -68,21 +74,28 @@ __global__ void __launch_bounds__(256) k_assemble_f64(Batch bt, const double* __
   const double ca = cos(alpha[b]), sa = sin(alpha[b]);
   double* Ab = A + bt.mat_off[b];
   double* rb = rhs + vec_off(bt, b);
-  for (int j = threadIdx.x; j < m; j += blockDim.x)
+  const int j1 = min(m, j0 + rows);
+  for (int j = j0 + threadIdx.x; j < j1; j += blockDim.x)
     rb[j] = (j < n) ? v * (mys[j] * ca - mxs[j] * sa) : 0.0;
 
+  // a warp takes 31 panels of a row at a time: lane l the distance to node i0 + l
+  // and, below lane 31, the panel from it to the next lane's node
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int j = warp; j < m; j += nw) {
+  const int ncb = (n + 30) / 31;
+  for (int t = warp; t < ncb * (j1 - j0); t += nw) {
+    const int j = j0 + t / ncb, i = 31 * (t % ncb) + lane;
     double* row = Ab + (int64_t)j * m;
-    if (j < n) {
-      const double px = mxs[j], py = mys[j];
-      for (int i = lane; i < n; i += 32)
-        row[i] = -panel_G_f64(px, py, xs[i], ys[i], txs[i], tys[i], Ls[i]);
-      if (lane == 0) row[n] = 1.0;
-    } else {
-      for (int i = lane; i < m; i += 32) row[i] = (i == 0 || i == n - 1) ? 1.0 : 0.0;
-    }
+    if (j == n) continue;
+    const int k = i < n ? i : (i == n ? 0 : n - 1);  // the node; x_n = x_0
+    const double dx = mxs[j] - xs[k], dy = mys[j] - ys[k];
+    const double la = log(dx * dx + dy * dy);
+    const double lb = __shfl_down_sync(0xffffffffu, la, 1);
+    if (lane < 31 && i < n) row[i] = -panel_G_f64(dx, dy, la, lb, txs[i], tys[i], Ls[i]);
   }
+  for (int j = j0 + threadIdx.x; j < min(j1, n); j += blockDim.x) Ab[(int64_t)j * m + n] = 1.0;
+  if (j1 == m)
+    for (int i = threadIdx.x; i < m; i += blockDim.x)
+      Ab[(int64_t)n * m + i] = (i == 0 || i == n - 1) ? 1.0 : 0.0;
 }
 
 size_t assemble_f64_smem(int n_max) { return (size_t)(7 * n_max + 32) * sizeof(double); }
@@ -92,7 +105,9 @@ cudaError_t launch_assemble_f64(const Batch& bt, const double* alpha, const doub
   size_t smem = assemble_f64_smem(bt.n_max);
   cudaError_t e = ensure_smem(k_assemble_f64, smem);
   if (e != cudaSuccess) return e;
-  k_assemble_f64<<<bt.B, 256, smem, s>>>(bt, alpha, vinf, A, rhs, info);
+  const int rows = f64_rows(bt.B, bt.n_max + 1);
+  k_assemble_f64<<<dim3(bt.B, (bt.n_max + rows) / rows), 256, smem, s>>>(bt, alpha, vinf, A, rhs,
+                                                                         info, rows);
   return cudaGetLastError();
 }
 

@@ -156,4 +156,15 @@ inline int sm_count() {
   return n;
 }
 
+// Rows per block of the plain FP64 pair kernels (launched for B airfoils of at most m
+// rows): all of them for a batch of four blocks per SM, else as few as spread the
+// batch over that many blocks, at least 12 (a block's own preparation costs about three
+// rows).
+inline int f64_rows(int B, int m) {
+  const long long want = 4ll * (sm_count() > 0 ? sm_count() : 1);
+  const long long z = (want + B - 1) / (B > 0 ? B : 1);
+  const long long rows = (m + z - 1) / z;
+  return (int)(rows < 12 ? (m < 12 ? m : 12) : rows);
+}
+
 }  // namespace panel

@@ -147,3 +147,49 @@ def test_cluster_refinement_with_the_inverse(n):
         out.append((pb.u.cpu().numpy(), pb.grad.cpu().numpy()))
     assert np.max(np.abs(out[0][0] - out[1][0])) <= 1e-11 * np.max(np.abs(out[0][0]))
     assert np.max(np.abs(out[0][1] - out[1][1])) <= 1e-10 * np.max(np.abs(out[0][1]))
+
+
+@pytest.mark.parametrize("n", [3, 30, 31, 32, 61, 62, 63, 64, 93, 127, 128, 158, 159, 160, 170])
+def test_fp64_path_at_the_edges_of_its_tiles(n):
+    """31-panel column blocks, row ranges, the matrix in shared memory or not: against
+    the oracle, and the transposed solve of panel_adjoint against panel_solve's."""
+    need_gpu()
+    import oracle
+    from paper_1511_02166_gb300.solver import PanelBatch
+    pop = _airfoils((n, max(3, n - 1), max(3, n // 2)), seed=n)
+    ref = oracle.evaluate_batch(pop.nodes, pop.offsets, pop.alpha)
+    pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, mode="fp64", bucket_width=None)
+    pb.run(with_grad=True)
+    assert int(pb.info.abs().max()) == 0
+    u, lam, g = (t.cpu().numpy() for t in (pb.u, pb.lam, pb.grad))
+    assert np.max(np.abs(u - ref["u"])) <= 1e-10 * np.max(np.abs(ref["u"]))
+    assert np.max(np.abs(pb.cl.cpu().numpy() - ref["cl"])) <= 1e-10
+    assert np.max(np.abs(pb.cl_p.cpu().numpy() - ref["cl_p"])) <= 1e-10
+    grad, _ = oracle.cl_gradient_batch(pop.nodes, pop.offsets, pop.alpha)
+    assert np.max(np.abs(g - grad)) <= 1e-9 * np.max(np.abs(grad))
+    pb.solve(with_adjoint=False)
+    pb.adjoint()
+    assert np.max(np.abs(pb.lam.cpu().numpy() - lam)) <= 1e-11 * np.max(np.abs(lam))
+
+
+@pytest.mark.parametrize("batch", [1, 609])
+@pytest.mark.parametrize("n", [3, 31, 33, 127, 129, 300])
+def test_forces_by_one_and_by_four_warps(batch, n):
+    """Cp, Cl and the pressure forces of both block shapes with vinf and chord given."""
+    need_gpu()
+    from paper_1511_02166_gb300.solver import PanelBatch
+    pop = _airfoils((n,), seed=n)
+    pop = inputs.pack([pop.airfoil(0)] * batch, np.tile(pop.alpha, batch))
+    v, c = np.full(batch, 1.7), np.full(batch, 0.9)
+    pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, vinf=v, chord=c, bucket_width=None)
+    pb.run()
+    x, a = pop.airfoil(batch - 1), pop.alpha[-1]
+    g = pb.gamma(batch - 1).cpu().numpy()
+    h = np.roll(x, -1, axis=0) - x
+    cp = 1 - (g / 1.7)**2
+    f = np.array([-(cp * h[:, 1]).sum(), (cp * h[:, 0]).sum()])
+    tol = 1e-13 * (1 + np.abs(cp).sum())
+    assert np.max(np.abs(pb.cp[-n:].cpu().numpy() - cp)) <= 1e-13 * np.max(np.abs(cp))
+    assert abs(float(pb.cl[-1]) - 2 * (g * np.hypot(*h.T)).sum() / (1.7 * 0.9)) <= tol
+    assert abs(float(pb.cl_p[-1]) - (-f[0] * np.sin(a) + f[1] * np.cos(a)) / 0.9) <= tol
+    assert abs(float(pb.cd_p[-1]) - (f[0] * np.cos(a) + f[1] * np.sin(a)) / 0.9) <= tol
