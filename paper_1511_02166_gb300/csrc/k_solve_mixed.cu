@@ -657,13 +657,13 @@ static size_t lu_global_smem(int n_max) {
 // one of them or both at once.  Both go over the 32-row groups of the factor
 // top-down (L, U^T) and then bottom-up (U, L^T), two block barriers per group:
 //   phase A  forward: t_i = y_i - (row i of L or U outside the group) . y, a
-//            warp per row, lanes along the row (left-looking, coalesced);
+//            few rows per warp, lanes along the rows (left-looking, coalesced);
 //            transposed: the previous group's columns of U^T (rows of U), or
 //            of L^T, applied to the rest of z, a thread per column
 //            (right-looking, coalesced across the threads); the group's own
 //            entries go to its 32-float scratch instead of z;
-//   phase B  the group's diagonal block: y_i = sum X_iq t_q (a warp per row),
-//            z_i = sum X_qi t_q (a warp per column).
+//   phase B  the group's diagonal block: y_i = sum X_iq t_q, z_i = sum X_qi t_q
+//            (a few rows / columns per warp).
 // Solving both systems, every warp takes its share of both in each phase (the
 // two share the barriers, and a warp done with its forward rows goes on to its
 // transposed columns while others are still loading); each system's
@@ -675,53 +675,95 @@ __device__ __forceinline__ float warp_sum_f(float v) {
   return v;
 }
 
-__device__ __forceinline__ float sum8(const float (&a)[8]) {
-  return ((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7]));
+// Sums over the lanes of R values per lane (R = 1, 2, 4, 8): log2 R halving exchanges
+// (each lane keeps half of the values and adds the partner's copies of them), then
+// butterflies; the total of value r is in the lanes l with l / (32 / R) == r.  R = 8
+// takes 9 shuffles instead of 40.
+template <int R>
+__device__ __forceinline__ float lane_sums(float (&v)[R], int lane) {
+  int o = 16;
+#pragma unroll
+  for (int h = R / 2; h >= 1; h >>= 1, o >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int r = 0; r < h; ++r) {
+      const float keep = up ? v[r + h] : v[r], send = up ? v[r] : v[r + h];
+      v[r] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  float s = v[0];
+#pragma unroll
+  for (int k = 16 / R; k >= 1; k >>= 1) s += __shfl_xor_sync(0xffffffffu, s, k);
+  return s;
 }
 
-// One lane's shares of sum_{k in [k0, k1)} row[k] y[k] (k = lane + 32 t) for
-// two rows r0 and r1 (r1 only if `two`) over the same columns, with eight
-// independent partial sums per row, so that up to sixteen loads are in flight
-// per lane (a long row is otherwise a chain of dependent round trips to L2);
-// the last (< 256) columns take one masked pass.
-__device__ __forceinline__ float2 row_dot2(const float* __restrict__ r0,
-                                           const float* __restrict__ r1, bool two,
-                                           const float* y, int k0, int k1, int lane) {
-  float a[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  float b[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  int k = k0 + lane;
-  for (; k + 7 * 32 < k1; k += 8 * 32) {
-    float u[8], v[8];
+// acc[r] += sum over the chunks c in [c0, c1) of p[r rs + c cs] y[32 c] for R rows (p and
+// y already offset by the lane): per chunk R loads, one shared read of y, R
+// multiply-adds; U chunks' loads in flight.
+template <int R, int U>
+__device__ __forceinline__ void rows_dot(float (&acc)[R], const float* __restrict__ p, int rs,
+                                         int cs, const float* y, int c0, int c1) {
+  int c = c0;
+  for (; c + U <= c1; c += U) {
+    float v[U][R];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      u[t] = __ldg(r0 + k + 32 * t);
-      v[t] = two ? __ldg(r1 + k + 32 * t) : 0.0f;
-    }
+    for (int u = 0; u < U; ++u)
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const float yy = y[k + 32 * t];
-      a[t] = fmaf(u[t], yy, a[t]);
-      b[t] = fmaf(v[t], yy, b[t]);
+      for (int r = 0; r < R; ++r) v[u][r] = __ldg(p + (c + u) * cs + r * rs);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float yy = y[32 * (c + u)];
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r] = fmaf(v[u][r], yy, acc[r]);
     }
   }
-  if (k < k1) {
-    float u[8], v[8];
+  if (U > 1)
+    for (; c < c1; ++c) {
+      const float yy = y[32 * c];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const bool ok = k + 32 * t < k1;
-      u[t] = ok ? __ldg(r0 + k + 32 * t) : 0.0f;
-      v[t] = (ok && two) ? __ldg(r1 + k + 32 * t) : 0.0f;
+      for (int r = 0; r < R; ++r) acc[r] = fmaf(__ldg(p + c * cs + r * rs), yy, acc[r]);
     }
+}
+
+// The same over the columns [c0, c1) of R rows stored row-major (stride m, from F):
+// full chunks, then one masked chunk.
+template <int R, int U>
+__device__ __forceinline__ void rows_dot_range(float (&acc)[R], const float* __restrict__ F, int m,
+                                               const float* y, int c0, int c1, int lane) {
+  const int full = (c1 - c0) >> 5;
+  rows_dot<R, U>(acc, F + c0 + lane, m, 32, y + c0 + lane, 0, full);
+  const int c = c0 + 32 * full + lane;
+  if (c < c1) {
+    const float yy = y[c];
 #pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      if (k + 32 * t < k1) {
-        const float yy = y[k + 32 * t];
-        a[t] = fmaf(u[t], yy, a[t]);
-        b[t] = fmaf(v[t], yy, b[t]);
+    for (int r = 0; r < R; ++r) acc[r] = fmaf(__ldg(F + c + r * m), yy, acc[r]);
+  }
+}
+
+// z -= the 32 (or kb) rows p, p + step, .. of a group, times the group's values g
+// (16-byte aligned), for one column.
+template <int U>
+__device__ __forceinline__ float column_update(const float* __restrict__ p, int step, int kb,
+                                               const float* g, float acc) {
+  if (kb == 32) {
+#pragma unroll 1
+    for (int t = 0; t < 32; t += U) {
+      float v[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) v[u] = __ldg(p + (t + u) * step);
+#pragma unroll
+      for (int u = 0; u < U; u += 4) {
+        const float4 q = *reinterpret_cast<const float4*>(g + t + u);
+        acc = fmaf(-v[u], q.x, acc);
+        acc = fmaf(-v[u + 1], q.y, acc);
+        acc = fmaf(-v[u + 2], q.z, acc);
+        acc = fmaf(-v[u + 3], q.w, acc);
       }
     }
+  } else {
+    for (int t = 0; t < kb; ++t) acc = fmaf(-__ldg(p + t * step), g[t], acc);
   }
-  return make_float2(sum8(a), sum8(b));
+  return acc;
 }
 
 // The factor of an airfoil of at most kLargeM - 1 panels: row-major, ld m,
@@ -732,24 +774,27 @@ struct RmFactor {
   __device__ int groups() const { return (m + 31) >> 5; }
   __device__ int k0(int d) const { return 32 * d; }
   __device__ int kb(int d) const { return min(32, m - 32 * d); }
-  // lane shares of row i . y (and of row i1 . y if `two`) over the columns
-  // before / after group d
-  __device__ float2 dot_left(int i, int i1, bool two, int d, const float* y, int lane) const {
-    return row_dot2(F + (int64_t)i * m, F + (int64_t)i1 * m, two, y, 0, 32 * d, lane);
+  // lane shares of rows i .. i + R - 1 (of group d) . y over the columns before /
+  // after the group; i + R - 1 may run past the group's (and the matrix's) last row:
+  // the caller asks for existing rows only (R full rows, or one at a time)
+  template <int R, int U>
+  __device__ void dot_left(float (&acc)[R], int i, int d, const float* y, int lane) const {
+    rows_dot<R, U>(acc, F + i * m + lane, m, 32, y + lane, 0, d);
   }
-  __device__ float2 dot_right(int i, int i1, bool two, int d, const float* y, int lane) const {
-    return row_dot2(F + (int64_t)i * m, F + (int64_t)i1 * m, two, y, 32 * d + kb(d), m, lane);
+  template <int R, int U>
+  __device__ void dot_right(float (&acc)[R], int i, int d, const float* y, int lane) const {
+    rows_dot_range<R, U>(acc, F + i * m, m, y, 32 * d + kb(d), m, lane);
   }
-  // row i's entries in the columns of group d
+  // row i's entries in the columns of group d, and the distance between rows
   __device__ const float* diag_row(int d, int i) const { return F + (int64_t)i * m + 32 * d; }
-  // z_r -= sum_t M[k0 + t][r] z_{k0 + t} (group d's rows) for the columns r after
-  // group d; those of group d + 1 go to nx.  Thread tid of nth.
-  __device__ void update_right(int d, float* z, float* nx, int tid, int nth) const {
+  __device__ int diag_step(int) const { return m; }
+  // z_r -= sum_t M[k0 + t][r] g_t (group d's rows, its values g) for the columns r
+  // after group d; those of group d + 1 go to nx.  Thread tid of nth.
+  template <int U>
+  __device__ void update_right(int d, float* z, const float* g, float* nx, int tid, int nth) const {
     const int k0 = 32 * d, kb = this->kb(d), c0 = k0 + kb;
     for (int r = c0 + tid; r < m; r += nth) {
-      float acc = z[r];
-#pragma unroll 8
-      for (int t = 0; t < kb; ++t) acc = fmaf(-__ldg(F + (int64_t)(k0 + t) * m + r), z[k0 + t], acc);
+      const float acc = column_update<U>(F + k0 * m + r, m, kb, g, z[r]);
       if (r < c0 + 32)
         nx[r - c0] = acc;
       else
@@ -757,12 +802,11 @@ struct RmFactor {
     }
   }
   // the same for the columns before group d; those of group d - 1 go to nx
-  __device__ void update_left(int d, float* z, float* nx, int tid, int nth) const {
+  template <int U>
+  __device__ void update_left(int d, float* z, const float* g, float* nx, int tid, int nth) const {
     const int k0 = 32 * d, kb = this->kb(d);
     for (int r = tid; r < k0; r += nth) {
-      float acc = z[r];
-#pragma unroll 8
-      for (int t = 0; t < kb; ++t) acc = fmaf(-__ldg(F + (int64_t)(k0 + t) * m + r), z[k0 + t], acc);
+      const float acc = column_update<U>(F + k0 * m + r, m, kb, g, z[r]);
       if (r >= k0 - 32)
         nx[r - (k0 - 32)] = acc;
       else
@@ -788,57 +832,14 @@ struct CrFactor;
 struct CrRag {
   const float* p;  // the block row's span
   int hh, e;
-  int64_t jump;    // the full tiles' floats
+  int jump;        // the full tiles' floats
   __device__ CrRag(const float* F, const TlGeom& g, int I)
-      : p(F + g.span(I)), hh(g.head(I)), e(g.e), jump((int64_t)(g.T - 1) * kTlTile) {}
+      : p(F + g.span(I)), hh(g.head(I)), e(g.e), jump((g.T - 1) * kTlTile) {}
   __device__ float operator()(int rr, int c) const {
     const int idx = rr * e + c;
-    return __ldg(p + (idx < hh ? (int64_t)idx : idx + jump));
+    return __ldg(p + (idx < hh ? idx : idx + jump));
   }
 };
-
-// sum_{ch in [c0, c1)} p[4096 ch] yy[32 ch] (one lane's share of a chunked row:
-// p and yy already offset by the lane) for two rows p0 and p1 (p1 only if
-// `two`), as row_dot2.
-__device__ __forceinline__ float2 chunk_dot2(const float* __restrict__ p0,
-                                             const float* __restrict__ p1, bool two,
-                                             const float* yy, int c0, int c1) {
-  float a[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  float b[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  int ch = c0;
-  for (; ch + 7 < c1; ch += 8) {
-    float u[8], v[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      u[t] = __ldg(p0 + (int64_t)(ch + t) * kTlChunk);
-      v[t] = two ? __ldg(p1 + (int64_t)(ch + t) * kTlChunk) : 0.0f;
-    }
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const float y = yy[32 * (ch + t)];
-      a[t] = fmaf(u[t], y, a[t]);
-      b[t] = fmaf(v[t], y, b[t]);
-    }
-  }
-  if (ch < c1) {
-    float u[8], v[8];
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      const bool ok = ch + t < c1;
-      u[t] = ok ? __ldg(p0 + (int64_t)(ch + t) * kTlChunk) : 0.0f;
-      v[t] = (ok && two) ? __ldg(p1 + (int64_t)(ch + t) * kTlChunk) : 0.0f;
-    }
-#pragma unroll
-    for (int t = 0; t < 8; ++t) {
-      if (ch + t < c1) {
-        const float y = yy[32 * (ch + t)];
-        a[t] = fmaf(u[t], y, a[t]);
-        b[t] = fmaf(v[t], y, b[t]);
-      }
-    }
-  }
-  return make_float2(sum8(a), sum8(b));
-}
 
 struct CrFactor {
   const float* F;  // the airfoil's matrix
@@ -860,45 +861,45 @@ struct CrFactor {
   __device__ const float* chunk_row(int I, int rr) const {
     return F + g.tile(I, 1) + (int64_t)rr * kTlC;
   }
-  // rows i and i1 (i1 only if `two`) of group d, as RmFactor
-  __device__ float2 dot_left(int i, int i1, bool two, int d, const float* y, int lane) const {
-    if (d < G0) return row_dot2(F + (int64_t)i * m, F + (int64_t)i1 * m, two, y, 0, 32 * d, lane);
-    const int e = g.e, I = 1 + ((i - e) >> 7), rr = (i - e) & (kTlB - 1), rr1 = (i1 - e) & (kTlB - 1);
-    const CrRag rag(F, g, I);
-    float v = 0.0f, w = 0.0f;
-#pragma unroll
-    for (int t = 0; t < kTlB / 32; ++t) {
-      const int c = lane + 32 * t;
-      if (c < e) {
-        v = fmaf(rag(rr, c), y[c], v);
-        if (two) w = fmaf(rag(rr1, c), y[c], w);
-      }
+  // rows i .. i + R - 1 of group d, as RmFactor
+  template <int R, int U>
+  __device__ void dot_left(float (&acc)[R], int i, int d, const float* y, int lane) const {
+    if (d < G0) {
+      rows_dot<R, U>(acc, F + i * m + lane, m, 32, y + lane, 0, d);
+      return;
     }
-    const float2 p = chunk_dot2(chunk_row(I, rr) + lane, chunk_row(I, rr1) + lane, two,
-                                y + e + lane, 0, d - G0);
-    return make_float2(v + p.x, w + p.y);
+    const int e = g.e, I = 1 + ((i - e) >> 7), rr = (i - e) & (kTlB - 1);
+    const CrRag rag(F, g, I);
+#pragma unroll 1
+    for (int c = lane; c < e; c += 32) {
+      const float yy = y[c];
+#pragma unroll
+      for (int r = 0; r < R; ++r) acc[r] = fmaf(rag(rr + r, c), yy, acc[r]);
+    }
+    rows_dot<R, U>(acc, chunk_row(I, rr) + lane, kTlC, kTlChunk, y + e + lane, 0, d - G0);
   }
-  __device__ float2 dot_right(int i, int i1, bool two, int d, const float* y, int lane) const {
-    if (d < G0)
-      return row_dot2(F + (int64_t)i * m, F + (int64_t)i1 * m, two, y, k0(d) + kb(d), m, lane);
-    const int e = g.e, I = 1 + ((i - e) >> 7), rr = (i - e) & (kTlB - 1), rr1 = (i1 - e) & (kTlB - 1);
-    return chunk_dot2(chunk_row(I, rr) + lane, chunk_row(I, rr1) + lane, two, y + e + lane,
-                      d - G0 + 1, nch);
+  template <int R, int U>
+  __device__ void dot_right(float (&acc)[R], int i, int d, const float* y, int lane) const {
+    if (d < G0) {
+      rows_dot_range<R, U>(acc, F + i * m, m, y, k0(d) + kb(d), m, lane);
+      return;
+    }
+    const int e = g.e, I = 1 + ((i - e) >> 7), rr = (i - e) & (kTlB - 1);
+    rows_dot<R, U>(acc, chunk_row(I, rr) + lane, kTlC, kTlChunk, y + e + lane, d - G0 + 1, nch);
   }
   __device__ const float* diag_row(int d, int i) const {
     if (d < G0) return F + (int64_t)i * m + 32 * d;
     const int h = d - G0, rr = (i - g.e) & (kTlB - 1);
     return chunk_row(1 + (h >> 2), rr) + (int64_t)h * kTlChunk;
   }
-  __device__ void update_right(int d, float* z, float* nx, int tid, int nth) const {
+  __device__ int diag_step(int d) const { return d < G0 ? m : kTlC; }
+  template <int U>
+  __device__ void update_right(int d, float* z, const float* gv, float* nx, int tid, int nth) const {
     const int k0 = this->k0(d), kb = this->kb(d), c0 = k0 + kb;
     const int c1 = c0 + this->kb(d + 1);  // end of group d + 1 (d + 1 < groups())
     if (d < G0) {
       for (int r = c0 + tid; r < m; r += nth) {
-        float acc = z[r];
-#pragma unroll 16
-        for (int t = 0; t < kb; ++t)
-          acc = fmaf(-__ldg(F + (int64_t)(k0 + t) * m + r), z[k0 + t], acc);
+        const float acc = column_update<U>(F + k0 * m + r, m, kb, gv, z[r]);
         if (r < c1)
           nx[r - c0] = acc;
         else
@@ -908,10 +909,8 @@ struct CrFactor {
       const int h = d - G0, e = g.e;
       const float* p = chunk_row(1 + (h >> 2), 32 * (h & 3));  // row k0 of the group
       for (int c = 32 * (h + 1) + tid; c < 32 * nch; c += nth) {
-        const float* pc = p + (int64_t)(c >> 5) * kTlChunk + (c & 31);
-        float acc = z[e + c];
-#pragma unroll 16
-        for (int t = 0; t < 32; ++t) acc = fmaf(-__ldg(pc + t * kTlC), z[k0 + t], acc);
+        const float* pc = p + (c >> 5) * kTlChunk + (c & 31);
+        const float acc = column_update<U>(pc, kTlC, 32, gv, z[e + c]);
         if (e + c < c1)
           nx[e + c - c0] = acc;
         else
@@ -919,15 +918,13 @@ struct CrFactor {
       }
     }
   }
-  __device__ void update_left(int d, float* z, float* nx, int tid, int nth) const {
+  template <int U>
+  __device__ void update_left(int d, float* z, const float* gv, float* nx, int tid, int nth) const {
     const int k0 = this->k0(d), kb = this->kb(d);
     const int p0 = this->k0(d - 1);  // start of group d - 1 (d >= 1)
     if (d < G0) {
       for (int r = tid; r < k0; r += nth) {
-        float acc = z[r];
-#pragma unroll 16
-        for (int t = 0; t < kb; ++t)
-          acc = fmaf(-__ldg(F + (int64_t)(k0 + t) * m + r), z[k0 + t], acc);
+        const float acc = column_update<U>(F + k0 * m + r, m, kb, gv, z[r]);
         if (r >= p0)
           nx[r - p0] = acc;
         else
@@ -940,7 +937,7 @@ struct CrFactor {
       for (int r = tid; r < e; r += nth) {
         float acc = z[r];
 #pragma unroll 16
-        for (int t = 0; t < 32; ++t) acc = fmaf(-rag(rr0 + t, r), z[k0 + t], acc);
+        for (int t = 0; t < 32; ++t) acc = fmaf(-rag(rr0 + t, r), gv[t], acc);
         if (r >= p0)
           nx[r - p0] = acc;
         else
@@ -949,10 +946,8 @@ struct CrFactor {
       // columns e .. k0 - 1: the chunks before the group's
       const float* p = chunk_row(I, rr0);
       for (int c = tid; c < 32 * h; c += nth) {
-        const float* pc = p + (int64_t)(c >> 5) * kTlChunk + (c & 31);
-        float acc = z[e + c];
-#pragma unroll 16
-        for (int t = 0; t < 32; ++t) acc = fmaf(-__ldg(pc + t * kTlC), z[k0 + t], acc);
+        const float* pc = p + (c >> 5) * kTlChunk + (c & 31);
+        const float acc = column_update<U>(pc, kTlC, 32, gv, z[e + c]);
         if (e + c >= p0)
           nx[e + c - p0] = acc;
         else
@@ -962,111 +957,118 @@ struct CrFactor {
   }
 };
 
-// FWD: y <- U^{-1} L^{-1} y (scratch ty); TRN: z <- L^{-T} U^{-T} z (scratch tz).
-template <bool FWD, bool TRN, class Fac>
+// FWD: y <- U^{-1} L^{-1} y (scratch ty, 32 floats); TRN: z <- L^{-T} U^{-T} z (scratch
+// tz, 64 floats, 16-byte aligned: the group's incoming values, then its results).
+// Each of the block's 32 / R warps takes R neighbouring rows (columns) of a group,
+// whose products share the reads of the vector and whose sums over the lanes are
+// taken together (lane_sums): with one row after the other, the sums, masks and
+// addresses were five times the instructions of the products, and the sweeps 61 % of
+// the refinement of 4096 x 200 panels.
+template <bool FWD, bool TRN, int R, class Fac>
 __device__ void lu_sweeps(const Fac& f, float* y, float* z, float* ty, float* tz) {
   static_assert(FWD || TRN, "a system to solve");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-  const int tid = (int)threadIdx.x, nt = (int)blockDim.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int tid = (int)threadIdx.x;
+  constexpr int NT = 1024 / R;
+  // loads in flight per lane: chunks of the rows (8 loads; 16 for the two rows of the
+  // largest airfoils' blocks, 14.9 -> 14.6 ms on 304 of 1024..2048), and entries of a
+  // column (8 where 8 blocks share an SM; 32 rather than 16 took 304 of 600 from 2022
+  // to 1929 us)
+  constexpr int U = R >= 8 ? 1 : R == 4 ? 2 : 16 / R;
+  constexpr int UC = R >= 8 ? 8 : 32;
   const int G = f.groups();
-  for (int d = 0; d < G; ++d) {
+  const int q0 = warp * R, sub = lane / (32 / R);  // the warp's rows; the lane's of them
+  float* gz = tz + 32;
+#pragma unroll 1
+  for (int s = 0; s < 2 * G; ++s) {
+    const bool down = s < G;
+    const int d = down ? s : 2 * G - 1 - s;
     const int k0 = f.k0(d), kb = f.kb(d);
     if (FWD) {
-      // rows q and q + nw of the group together
-      for (int q = warp; q < kb; q += 2 * nw) {
-        const int i = k0 + q, q1 = q + nw;
-        const bool two = q1 < kb;
-        const float2 p = f.dot_left(i, two ? k0 + q1 : i, two, d, y, lane);
-        const float acc = warp_sum_f(p.x), acc1 = warp_sum_f(p.y);
-        if (lane == 0) {
-          ty[q] = y[i] - acc;
-          if (two) ty[q1] = y[k0 + q1] - acc1;
+      // t = y - (rows of L left of the group, of U right of it) . y
+      if (q0 + R <= kb) {
+        float acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = 0.0f;
+        if (down)
+          f.template dot_left<R, U>(acc, k0 + q0, d, y, lane);
+        else
+          f.template dot_right<R, U>(acc, k0 + q0, d, y, lane);
+        const float v = lane_sums<R>(acc, lane);
+        if ((lane & (32 / R - 1)) == 0) ty[q0 + sub] = y[k0 + q0 + sub] - v;
+      } else {
+        for (int q = q0; q < kb; ++q) {  // the last rows of a short group
+          float acc[1] = {0.0f};
+          if (down)
+            f.template dot_left<1, 1>(acc, k0 + q, d, y, lane);
+          else
+            f.template dot_right<1, 1>(acc, k0 + q, d, y, lane);
+          const float v = warp_sum_f(acc[0]);
+          if (lane == 0) ty[q] = y[k0 + q] - v;
         }
       }
     }
     if (TRN) {
-      if (d == 0) {
+      if (s == 0 || s == G) {
         if (tid < 32) tz[tid] = (tid < kb) ? z[k0 + tid] : 0.0f;
+      } else if (down) {
+        f.template update_right<UC>(d - 1, z, gz, tz, tid, NT);
       } else {
-        f.update_right(d - 1, z, tz, tid, nt);
+        f.template update_left<UC>(d + 1, z, gz, tz, tid, NT);
       }
     }
     __syncthreads();
     if (FWD) {
-      for (int q = warp; q < kb; q += nw) {
-        const int i = k0 + q;
-        // y_i = t_i + sum_{k<i} X[i][k] t_k  (X unit lower, stored below the diagonal)
-        float v = (lane < q) ? __ldg(f.diag_row(d, i) + lane) * ty[lane] : 0.0f;
-        v = warp_sum_f(v);
-        if (lane == 0) y[i] = ty[q] + v;
+      // down: y_i = t_i + sum_{k<i} X[i][k] t_k (X unit lower, stored below the
+      // diagonal); up: y_i = sum_{k>=i} Y[i][k] t_k (Y upper with diagonal)
+      const float t = (lane < kb) ? ty[lane] : 0.0f;
+      const float* p = f.diag_row(d, k0) + lane;
+      const int step = f.diag_step(d);
+      float v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int q = q0 + r;
+        const bool on = q < kb && lane < kb && (down ? lane < q : lane >= q);
+        v[r] = on ? __ldg(p + q * step) * t : 0.0f;
       }
+      const float w = lane_sums<R>(v, lane);
+      const int q = q0 + sub;
+      if ((lane & (32 / R - 1)) == 0 && q < kb) y[k0 + q] = down ? ty[q] + w : w;
     }
     if (TRN) {
-      for (int q = warp; q < kb; q += nw) {
-        // z_i = sum_{k<=i} Y[k][i] t_k  (Y upper with diagonal)
-        const int i = k0 + q;
-        float v = (lane <= q) ? __ldg(f.diag_row(d, k0 + lane) + q) * tz[lane] : 0.0f;
-        v = warp_sum_f(v);
-        if (lane == 0) z[i] = v;
+      // down: z_i = sum_{k<=i} Y[k][i] t_k; up: z_i = t_i + sum_{k>i} X[k][i] t_k
+      const float t = (lane < kb) ? tz[lane] : 0.0f;
+      const float* p = f.diag_row(d, k0) + lane * f.diag_step(d);
+      float v[R];
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int q = q0 + r;
+        const bool on = q < kb && lane < kb && (down ? lane <= q : lane > q);
+        v[r] = on ? __ldg(p + q) * t : 0.0f;
       }
-    }
-    __syncthreads();
-  }
-  for (int d = G - 1; d >= 0; --d) {
-    const int k0 = f.k0(d), kb = f.kb(d);
-    if (FWD) {
-      for (int q = warp; q < kb; q += 2 * nw) {
-        const int i = k0 + q, q1 = q + nw;
-        const bool two = q1 < kb;
-        const float2 p = f.dot_right(i, two ? k0 + q1 : i, two, d, y, lane);
-        const float acc = warp_sum_f(p.x), acc1 = warp_sum_f(p.y);
-        if (lane == 0) {
-          ty[q] = y[i] - acc;
-          if (two) ty[q1] = y[k0 + q1] - acc1;
-        }
-      }
-    }
-    if (TRN) {
-      if (d == G - 1) {
-        if (tid < 32) tz[tid] = (tid < kb) ? z[k0 + tid] : 0.0f;
-      } else {
-        f.update_left(d + 1, z, tz, tid, nt);
-      }
-    }
-    __syncthreads();
-    if (FWD) {
-      for (int q = warp; q < kb; q += nw) {
-        const int i = k0 + q;
-        // y_i = sum_{k>=i} Y[i][k] t_k  (Y upper with diagonal)
-        float v = (lane >= q && lane < kb) ? __ldg(f.diag_row(d, i) + lane) * ty[lane] : 0.0f;
-        v = warp_sum_f(v);
-        if (lane == 0) y[i] = v;
-      }
-    }
-    if (TRN) {
-      for (int q = warp; q < kb; q += nw) {
-        // z_i = t_i + sum_{k>i} X[k][i] t_k  (X unit lower, stored below the diagonal)
-        const int i = k0 + q;
-        float v = (lane > q && lane < kb) ? __ldg(f.diag_row(d, k0 + lane) + q) * tz[lane] : 0.0f;
-        v = warp_sum_f(v);
-        if (lane == 0) z[i] = tz[q] + v;
+      const float w = lane_sums<R>(v, lane);
+      const int q = q0 + sub;
+      if ((lane & (32 / R - 1)) == 0 && q < kb) {
+        const float zi = down ? w : tz[q] + w;
+        z[k0 + q] = zi;
+        gz[q] = zi;
       }
     }
     __syncthreads();
   }
 }
 
-// The forward system (fw), the transposed one (tr) or both; ty, tz: 32 floats
-// each.  Both at once (COMBINE) or one after the other.
-template <bool COMBINE, class Fac>
+// The forward system (fw), the transposed one (tr) or both; ty: 32 floats, tz: 64.
+// Both at once (COMBINE) or one after the other.
+template <bool COMBINE, int R, class Fac>
 __device__ void lu_solve(const Fac& f, bool fw, bool tr, float* y, float* z, float* ty,
                          float* tz) {
   if (COMBINE && fw && tr) {
-    lu_sweeps<true, true>(f, y, z, ty, tz);
+    lu_sweeps<true, true, R>(f, y, z, ty, tz);
     return;
   }
-  if (fw) lu_sweeps<true, false>(f, y, z, ty, tz);
-  if (tr) lu_sweeps<false, true>(f, y, z, ty, tz);
+  if (fw) lu_sweeps<true, false, R>(f, y, z, ty, tz);
+  if (tr) lu_sweeps<false, true, R>(f, y, z, ty, tz);
 }
 
 // ---------------------------------------------------------------------------
@@ -1651,11 +1653,11 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
       if (run1) gj_apply_transposed(F, m, z, part);
     } else if constexpr (!KEEP) {
       if (cr)
-        lu_solve<true>(crf, run0, run1, y, z, t32, t32z);
+        lu_solve<true, 1024 / NT>(crf, run0, run1, y, z, t32, t32z);
       else
-        lu_solve<true>(RmFactor{F, m}, run0, run1, y, z, t32, t32z);
+        lu_solve<true, 1024 / NT>(RmFactor{F, m}, run0, run1, y, z, t32, t32z);
     } else {
-      lu_solve<false>(RmFactor{F, m}, run0, run1, y, z, t32, t32z);
+      lu_solve<false, 1024 / NT>(RmFactor{F, m}, run0, run1, y, z, t32, t32z);
     }
     for (int q = 0; q < 2; ++q) {
       if (!(q == 0 ? run0 : run1)) continue;
@@ -1903,16 +1905,18 @@ static int ir_cluster_capacity(int C) {
 }
 
 // Blocks per airfoil of a refinement by clusters, or 0 for k_ir_mixed: the most that
-// let every airfoil of the batch run at once.  Measured, both systems (us, k_ir_mixed /
-// clusters of 1, 2, 4, 8): 1 airfoil of 100 panels 126 / 134, 128, 124, 126; of 160
-// 223 / 200, 182, 175, 173; of 600 1370 / 996, 711, 587, 544; of 1024 4284 / 3581,
-// 2444, 1589, 1337; of 2048 11315 / 13937, 8303, 5719, 3578; 76 airfoils of 300 569 /
-// 411, 338; of 1024 7083 / 4802, 3210; 18 of 2048 14263 / 15700, 9393, 6256.
+// let every airfoil of the batch run at once.  Measured, both systems (us, the best
+// block shape of k_ir_mixed / clusters): 1 airfoil of 200 panels 169 / 203; of 256 228 /
+// 257; of 300 324 / 295 (8 blocks); of 600 797 / 577; of 1024 3581 (one block of 1024
+// threads) / 2444, 1589, 1310 (2, 4, 8); of 2048 11315 / 8303, 5719, 3521; 76 airfoils
+// of 300 335 / 348 (2); of 600 954 / 868 (2); of 1024 4802 / 3084 (2); 18 of 2048 14263
+// / 15700, 9393, 6006 (1, 2, 4).
 static int ir_cluster_blocks(const SolveArgs& a) {
   const int mv = a.bt.n_max + 1;
-  if (a.ir_shape != 0 || mv <= 128) return 0;
+  if (a.ir_shape != 0 || mv <= kFuseM) return 0;
   for (int C = 8; C >= 1; C >>= 1)
-    if (a.bt.B <= ir_cluster_capacity(C)) return (C == 1 && mv > 1400) ? 0 : C;
+    if (a.bt.B <= ir_cluster_capacity(C))
+      return ((C < 4 && mv <= 400) || (C == 1 && mv > 1400)) ? 0 : C;
   return 0;
 }
 
@@ -1948,6 +1952,13 @@ static cudaError_t launch_ir_kernel(const SolveArgs& a, cudaStream_t s) {
     default:
       break;
   }
+  // few airfoils per SM: more warps for each (us, both systems, 256 x 4 / 512 x 2 / 256 x
+  // 3: 1 of 100 panels 90 / 87 / 85, 152 of 160 154 / 138 / 142, 304 of 200 283 / 279 /
+  // 257, 608 of 256 644 / 790 / 702, 76 of 300 410 / 322 / 397)
+  const int sms = sm_count(), mv = n_max + 1;
+  if (fits(512, 2) && ((mv > 128 && a.bt.B <= sms) || (mv > kFuseM && a.bt.B <= 2 * sms)))
+    return launch_ir_shape<512, 2>(a, s);
+  if (mv <= kFuseM && a.bt.B <= 3 * sms) return launch_ir_shape<kThreads, 3>(a, s);
   if (fits(128, 8) && n_max + 1 <= 7 * 32 && a.bt.B >= 8 * sm_count())
     return launch_ir_shape<128, 8, 7>(a, s);
   if (n_max + 1 <= kFuseM || fits(kThreads, 4)) return launch_ir_shape<kThreads, 4>(a, s);
