@@ -212,57 +212,121 @@ __device__ __forceinline__ void tri_subst(float (&x)[32], const DiagTab& d, cons
 // vector loads), the row exchanges, U12 and the rank-32 update applied to the
 // factor in the caller's LU buffer through L2.  Shared memory stays small (the
 // panel plus a 128-column slab of U12), so several airfoils share an SM and
-// hide each other's latencies.
+// hide each other's latencies.  A step has two phases:
+//   A  a warp per 32 rows: the panel's tile in, L21, and out to the factor; a
+//      warp per 32 columns: U12, the first slab of it kept for the update; the
+//      inverses of the diagonal block's triangles; the exchanges to the left;
+//   B  warp 0 updates the next diagonal block and factors it (look-ahead) while
+//      the others update everything else.
+// The first step reads the hi plane and writes the factor.  What bounded the
+// kernel were its chains of L2 and DRAM round trips, not the products: a copy of
+// the plane ahead of the first step, one load after the other, was 27-30 % of its
+// time, the unhidden diagonal blocks 28 % (201 unknowns) to 8 % (601), and moving
+// the panel between barriers of its own another 8-15 %.
 // ---------------------------------------------------------------------------
 constexpr int kSlabW = 128;  // columns of U12 staged at a time
 
-// A22 -= L21 U12 over the columns [cc, cc + 32 J) of the staged U12 slab: warp
-// w takes the 8-row tiles w, w + 8, ...; lane l the columns cc + l + 32 j.  lt:
-// row k1 of the transposed panel.
+// What a step reads the trailing matrix from: the factor, or (first step) the hi
+// plane, whose border the reader then scales by sf (after all of its loads: a
+// choice per load waits for each).
+struct LuSource {
+  const float* p;
+  int m;
+  float sf;
+  bool first;
+  __device__ __forceinline__ float operator()(int r, int c) const { return p[r * m + c]; }
+  __device__ __forceinline__ void scale(float& v, int r, int c) const {
+    if (r == m - 1 || c == m - 1) v *= sf;
+  }
+};
+
+// (d.x, d.y) + a (b, b), each rounded once.
+__device__ __forceinline__ void fma2(float2& d, float ax, float ay, float b) {
+  asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %4};\n\t"
+      "mov.b64 d, {%0, %1};\n\tfma.rn.f32x2 d, a, b, d;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "+f"(d.x), "+f"(d.y)
+      : "f"(ax), "f"(ay), "f"(b));
+}
+
+// A22 -= L21 U12 over the columns [cc, cc + 32 J) of the staged slab of -U12: the w-th
+// of nw warps takes the 8-row tiles w, w + nw, ...; lane l the columns cc + l + 32 j.
+// lt: row k1 of the transposed panel.  The next diagonal block (rows and columns
+// below k2) is warp 0's.
 template <int J>
-__device__ __forceinline__ void update_tiles(float* __restrict__ F, const float* __restrict__ lt,
-                                             int ldt, const float* __restrict__ U, int m, int k1,
-                                             int cc, int nrt) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int rt = warp; rt < nrt; rt += kWarps) {
-    const int r0 = k1 + 8 * rt;
-    float acc[8][J];
+__device__ __forceinline__ void update_tiles(const LuSource& S, float* F,
+                                             const float* __restrict__ lt, int ldt,
+                                             const float* __restrict__ U, int k1, int k2, int cc,
+                                             int nrt, int w, int nw) {
+  constexpr int R = 8;
+  const int lane = threadIdx.x & 31, m = S.m;
+  for (int rt = w; rt < nrt; rt += nw) {
+    const int r0 = k1 + R * rt;
+    float2 acc[R / 2][J];
 #pragma unroll
-    for (int aa = 0; aa < 8; ++aa)
+    for (int aa = 0; aa < R; ++aa)
 #pragma unroll
       for (int j = 0; j < J; ++j) {
         const int r = r0 + aa, c = cc + lane + 32 * j;
-        acc[aa][j] = (r < m && c < m) ? F[r * m + c] : 0.0f;
+        const float v = (r < m && c < m) ? S(r, c) : 0.0f;
+        if (aa & 1)
+          acc[aa / 2][j].y = v;
+        else
+          acc[aa / 2][j].x = v;
       }
-    const float* l0 = lt + 8 * rt;
-#pragma unroll 4
+    if (S.first)
+#pragma unroll
+      for (int aa = 0; aa < R; ++aa)
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+          S.scale((aa & 1) ? acc[aa / 2][j].y : acc[aa / 2][j].x, r0 + aa, cc + lane + 32 * j);
+    const float* l0 = lt + R * rt;
+#pragma unroll 2
     for (int q = 0; q < 32; ++q) {
-      const float4 la = *reinterpret_cast<const float4*>(l0 + q * ldt);
-      const float4 lb = *reinterpret_cast<const float4*>(l0 + q * ldt + 4);
-      const float lv[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
       float uv[J];
 #pragma unroll
       for (int j = 0; j < J; ++j) uv[j] = U[q * kSlabW + lane + 32 * j];
 #pragma unroll
-      for (int aa = 0; aa < 8; ++aa)
+      for (int a4 = 0; a4 < R / 4; ++a4) {
+        const float4 l = *reinterpret_cast<const float4*>(l0 + q * ldt + 4 * a4);
 #pragma unroll
-        for (int j = 0; j < J; ++j) acc[aa][j] = fmaf(-lv[aa], uv[j], acc[aa][j]);
+        for (int j = 0; j < J; ++j) {
+          fma2(acc[2 * a4][j], l.x, l.y, uv[j]);
+          fma2(acc[2 * a4 + 1][j], l.z, l.w, uv[j]);
+        }
+      }
     }
+    const int c0 = r0 < k2 ? k2 : 0;
 #pragma unroll
-    for (int aa = 0; aa < 8; ++aa)
+    for (int aa = 0; aa < R; ++aa)
 #pragma unroll
       for (int j = 0; j < J; ++j) {
         const int r = r0 + aa, c = cc + lane + 32 * j;
-        if (r < m && c < m) F[r * m + c] = acc[aa][j];
+        if (r < m && c < m && c >= c0) F[r * m + c] = (aa & 1) ? acc[aa / 2][j].y : acc[aa / 2][j].x;
       }
   }
 }
 
-// Row stride of the transposed panel: rows padded to whole 8-row tiles, and 4
-// mod 32, so that 4 rows x 8 columns moved by a warp touch all banks.
-__host__ __device__ constexpr int lu_panel_ld(int m) { return ((m + 8 + 31) & ~31) + 4; }
+// Row stride of the transposed panel: the rows below the first block, padded to
+// whole 8-row tiles and to whole 32-row tiles of phase A, and 4 mod 32, so that 4
+// rows x 8 columns moved by a warp touch all banks.
+__host__ __device__ constexpr int lu_panel_ld(int m) {
+  return (((m > 32 ? m - 32 : 1) + 31) & ~31) + 4;
+}
 
-__global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
+// Barriers of k_lu_global's phase B: the seven updating warps among themselves, and
+// (arrive / sync) warp 0's last read of the first slab.
+__device__ __forceinline__ void lu_update_sync() {
+  asm volatile("bar.sync 1, %0;\n" ::"n"(kThreads - 32) : "memory");
+}
+__device__ __forceinline__ void lu_slab_read() {
+  asm volatile("bar.arrive 2, %0;\n" ::"n"(kThreads) : "memory");
+}
+__device__ __forceinline__ void lu_slab_wait() {
+  asm volatile("bar.sync 2, %0;\n" ::"n"(kThreads) : "memory");
+}
+
+template <int MINB>
+__global__ void __launch_bounds__(kThreads, MINB) k_lu_global(SolveArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int NB = 32;
   const Batch& bt = a.bt;
@@ -283,37 +347,34 @@ __global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
   double* red = reinterpret_cast<double*>(U + NB * kSlabW);      // 32
   float* PT = reinterpret_cast<float*>(red + 32);                // NB x ldt panel, transposed
   const int ldt = lu_panel_ld(mv);
-  int* ipiv = reinterpret_cast<int*>(PT + NB * ldt);             // mv
+  float* D = PT + NB * ldt;                                      // NB x 33 diagonal block
+  int* ipiv = reinterpret_cast<int*>(D + NB * 33);               // mv
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int64_t moff = bt.mat_off[b];
   const float* Ah = a.A_hi + moff;
   float* F = a.LU + moff;
   diag_tab_init(dt);
-  const float sf = (float)border_scale(Ah, n, m, red);
-  for (int rr = warp; rr < m; rr += kWarps)
-    for (int cc = lane; cc < m; cc += 32) {
-      const float v = Ah[rr * m + cc];
-      F[rr * m + cc] = ((cc == n && rr < n) || rr == n) ? v * sf : v;
+  LuSource S{Ah, m, (float)border_scale(Ah, n, m, red), true};
+  auto diag = [&](int k, int kb) {
+    diag_lu([&](int r, int t) -> float& { return D[r * 33 + t]; }, kb, ipiv + k, k, dt);
+  };
+  if (warp == 0) {
+    const int kb = min(NB, m);
+#pragma unroll
+    for (int r = 0; r < NB; ++r)
+      if (r < kb && lane < kb) D[r * 33 + lane] = S(r, lane);
+    if (m <= NB && lane < m) {  // the block holds the border
+      D[n * 33 + lane] *= S.sf;
+      if (lane < n) D[lane * 33 + n] *= S.sf;
     }
+    __syncwarp();
+    diag(0, kb);
+  }
   __syncthreads();
 
   const int pc = lane & 7, pr = lane >> 3;  // panel moves: 8 columns x 4 rows per warp
-  for (int k0 = 0; k0 < m; k0 += NB) {
-    const int kb = min(NB, m - k0);
-    const int rows = m - k0;
-    // ---- stage the panel ----
-    for (int r = 4 * warp + pr; r < rows; r += 4 * kWarps)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int t = 8 * i + pc;
-        if (t < kb) PT[t * ldt + r] = F[(k0 + r) * m + k0 + t];
-      }
-    __syncthreads();
-    // ---- LU of the diagonal block by warp 0 (pivot search inside the block) ----
-    if (warp == 0)
-      diag_lu([&](int r, int t) -> float& { return PT[t * ldt + r]; }, kb, ipiv + k0, k0, dt);
-    __syncthreads();
+  for (int k0 = 0;; k0 += NB) {
     if (dt.fz != 0) {
       if (tid == 0) {
         a.info[b] = k0 + dt.fz;
@@ -321,8 +382,9 @@ __global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
       }
       return;
     }
+    const int kb = min(NB, m - k0);
     const int k1 = k0 + kb;
-    // ---- L21 = A21 U11^{-1}, a row per thread, in place in PT; U12 = L11^{-1}
+    // ---- A: L21 = A21 U11^{-1}, a row per thread, in place in PT; U12 = L11^{-1}
     // A12, a column per thread, the rows read through the block's exchanges; and
     // the two inverses of the diagonal block the refinement takes, U11^{-1} as 32
     // more rows (of the identity) and L11^{-1} as 32 more columns.  A warp takes
@@ -345,21 +407,43 @@ __global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
           if (q < kb && q > lane) G[q * m] = v;
         });
       } else if (w < 2 + nw) {
-        const int r = kb + 32 * (w - 2) + lane;
-        const bool ok = r < rows;
+        // the tile in, 32 loads a lane in flight, through the warp's own part of PT
+        const int rw = 32 * (w - 2);
+        float* T = PT + rw;
 #pragma unroll
-        for (int t = 0; t < 32; ++t) x[t] = ok ? PT[t * ldt + r] : 0.0f;
-        tri_subst<true>(x, dt, [&](int q, float v) {
-          if (ok) PT[q * ldt + r] = v;
-        });
+        for (int i = 0; i < 32; ++i) {
+          const int r = 4 * (i >> 2) + pr, t = 8 * (i & 3) + pc;
+          x[i] = (k1 + rw + r < m) ? S(k1 + rw + r, k0 + t) : 0.0f;
+        }
+        if (S.first)
+#pragma unroll
+          for (int i = 0; i < 32; ++i)
+            S.scale(x[i], k1 + rw + 4 * (i >> 2) + pr, k0 + 8 * (i & 3) + pc);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) T[(8 * (i & 3) + pc) * ldt + 4 * (i >> 2) + pr] = x[i];
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < 32; ++t) x[t] = T[t * ldt + lane];
+        tri_subst<true>(x, dt, [&](int q, float v) { T[q * ldt + lane] = v; });
+        __syncwarp();
+        float* G = F + (k1 + rw) * m + k0;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const int r = 4 * (i >> 2) + pr, t = 8 * (i & 3) + pc;
+          if (k1 + rw + r < m) G[r * m + t] = T[t * ldt + r];
+        }
       } else {
-        const int c = k1 + 32 * (w - 2 - nw) + lane;
-        const bool ok = c < m;
+        const int cu = 32 * (w - 2 - nw) + lane, c = k1 + cu;
+        const bool ok = c < m, slab = cu < kSlabW;
 #pragma unroll
-        for (int t = 0; t < 32; ++t) x[t] = ok ? F[(k0 + dt.bperm[t]) * m + c] : 0.0f;
+        for (int t = 0; t < 32; ++t) x[t] = ok ? S(k0 + dt.bperm[t], c) : 0.0f;
+        if (S.first && c == n)  // (the block's rows are not the last one)
+#pragma unroll
+          for (int t = 0; t < 32; ++t) x[t] *= S.sf;
         float* G = F + k0 * m + c;
         tri_subst<false>(x, dt, [&](int q, float v) {
           if (ok) G[q * m] = v;
+          if (slab) U[q * kSlabW + cu] = -v;
         });
       }
     }
@@ -376,32 +460,65 @@ __global__ void __launch_bounds__(kThreads, 3) k_lu_global(SolveArgs a) {
       }
     __syncthreads();
     if (k1 >= m) break;
-    // ---- L21 back to the factor ----
-    for (int r = kb + 4 * warp + pr; r < rows; r += 4 * kWarps)
+    // ---- B: A22 -= L21 U12, 128-column slabs of U12 staged in shared memory (the
+    // first one is there) ----
+    const int k2 = min(k1 + NB, m);
+    if (warp == 0) {
+      const int kb2 = k2 - k1;
+      float x[32];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) F[(k0 + r) * m + k0 + 8 * i + pc] = PT[(8 * i + pc) * ldt + r];
-    // ---- A22 -= L21 U12, 128-column slabs of U12 staged in shared memory ----
-    const int nrt = (m - k1 + 7) >> 3;
-    for (int cc = k1; cc < m; cc += kSlabW) {
-      for (int t = warp; t < kb; t += kWarps)
+      for (int r = 0; r < NB; ++r) x[r] = (r < kb2 && lane < kb2) ? S(k1 + r, k1 + lane) : 0.0f;
+      if (S.first)
 #pragma unroll
-        for (int j = 0; j < kSlabW / 32; ++j) {
-          const int c = cc + lane + 32 * j;
-          U[t * kSlabW + lane + 32 * j] = (c < m) ? F[(k0 + t) * m + c] : 0.0f;
+        for (int r = 0; r < NB; ++r) S.scale(x[r], k1 + r, k1 + lane);
+#pragma unroll 2
+      for (int q = 0; q < NB; ++q) {
+        const float uq = U[q * kSlabW + lane];
+#pragma unroll
+        for (int r4 = 0; r4 < 8; ++r4) {
+          const float4 l = *reinterpret_cast<const float4*>(PT + q * ldt + 4 * r4);
+          x[4 * r4] = fmaf(l.x, uq, x[4 * r4]);
+          x[4 * r4 + 1] = fmaf(l.y, uq, x[4 * r4 + 1]);
+          x[4 * r4 + 2] = fmaf(l.z, uq, x[4 * r4 + 2]);
+          x[4 * r4 + 3] = fmaf(l.w, uq, x[4 * r4 + 3]);
         }
-      __syncthreads();
-      // register tiles 8 rows x 32 J columns, J = 1..4 by the width of the slab
-      const int J = min(kSlabW / 32, (m - cc + 31) >> 5);
-      if (J == 4)
-        update_tiles<4>(F, PT + kb, ldt, U, m, k1, cc, nrt);
-      else if (J == 3)
-        update_tiles<3>(F, PT + kb, ldt, U, m, k1, cc, nrt);
-      else if (J == 2)
-        update_tiles<2>(F, PT + kb, ldt, U, m, k1, cc, nrt);
-      else
-        update_tiles<1>(F, PT + kb, ldt, U, m, k1, cc, nrt);
-      __syncthreads();
+      }
+      lu_slab_read();
+#pragma unroll
+      for (int r = 0; r < NB; ++r) D[r * 33 + lane] = x[r];
+      __syncwarp();
+      diag(k1, kb2);
+    } else {
+      const int nrt = k2 < m ? (m - k1 + 7) >> 3 : 0;
+      for (int cc = k1; cc < m; cc += kSlabW) {
+        if (cc > k1) {
+          for (int t = warp - 1; t < NB; t += kWarps - 1)
+#pragma unroll
+            for (int j = 0; j < kSlabW / 32; ++j) {
+              const int c = cc + lane + 32 * j;
+              U[t * kSlabW + lane + 32 * j] = (c < m) ? -F[(k0 + t) * m + c] : 0.0f;
+            }
+          lu_update_sync();
+        }
+        // register tiles 8 rows x 32 J columns, J = 1..4 by the width of the slab
+        const int J = min(kSlabW / 32, (m - cc + 31) >> 5);
+        if (J == 4)
+          update_tiles<4>(S, F, PT, ldt, U, k1, k2, cc, nrt, warp - 1, kWarps - 1);
+        else if (J == 3)
+          update_tiles<3>(S, F, PT, ldt, U, k1, k2, cc, nrt, warp - 1, kWarps - 1);
+        else if (J == 2)
+          update_tiles<2>(S, F, PT, ldt, U, k1, k2, cc, nrt, warp - 1, kWarps - 1);
+        else
+          update_tiles<1>(S, F, PT, ldt, U, k1, k2, cc, nrt, warp - 1, kWarps - 1);
+        if (cc == k1)
+          lu_slab_wait();
+        else
+          lu_update_sync();
+      }
     }
+    S.p = F;
+    S.first = false;
+    __syncthreads();
   }
   int32_t* gpiv = a.piv + vec_off(bt, b);
   for (int k = tid; k < m; k += kThreads) gpiv[k] = ipiv[k];
@@ -647,7 +764,7 @@ static size_t lu_smem_smem(int n_max) {
 static size_t lu_global_smem(int n_max) {
   const size_t mv = (size_t)n_max + 1;
   return sizeof(DiagTab) + 32 * (size_t)kSlabW * 4 + 32 * 8 +
-         32 * (size_t)lu_panel_ld((int)mv) * 4 + mv * 4;
+         32 * (size_t)lu_panel_ld((int)mv) * 4 + 32 * 33 * 4 + mv * 4;
 }
 
 // ---------------------------------------------------------------------------
@@ -1781,18 +1898,17 @@ static SolveArgs make_args(const Batch& bt, const float* A_hi, const float* A_lo
 }
 
 // Which one-block LU a launch of B airfoils of at most mv unknowns takes (1 through
-// L2, 2 in shared memory).  Up to 128 unknowns several airfoils of the
-// shared-memory form fit an SM and it is the faster one at any batch (4096 of 100
-// panels: 531 us against 727; one: 45 / 62).  Above, one airfoil fills the SM's
-// shared memory: it wins by its shorter steps until three L2-resident airfoils
-// per SM hide each other's (160 panels: 1 airfoil 70 / 116 us, 304 138 / 138, 1216
-// 552 / 523; 200 panels: 1 93 / 161, 304 185 / 218, 1216 745 / 789, 4096 2478 /
-// 2321).  A launch that also holds larger airfoils runs them all through L2 at
-// once.
+// L2, 2 in shared memory).  Up to 64 unknowns the shared-memory form's blocks of 128
+// threads, five on an SM, are the faster ones for any batch beyond three airfoils per
+// SM (4096 of 40 panels 145 us against 214; one 21 / 21).  Above, one to three of its
+// airfoils fit an SM and the L2-resident form is as fast or faster (4096 of 80 panels
+// 379 / 376, 128 1431 / 703, 205 2501 / 1557), but for a single airfoil per SM above
+// 160 unknowns, by its shorter steps (1 of 165 panels 69 / 72, of 205 91 / 98; 304 of
+// 165 141 / 93).  A launch that also holds larger airfoils runs them all through L2
+// at once.
 static int lu_kind_by_size(int B, int mv) {
   if (mv > kSmemLuM) return 1;
-  if (mv <= 128) return 2;
-  return B <= (mv <= 180 ? 2 : 12) * sm_count() ? 2 : 1;
+  return mv <= 64 || (mv > 160 && B <= sm_count()) ? 2 : 1;
 }
 
 // Factor every airfoil: with `inverse` the Gauss-Jordan inverse for m <= kGjM;
@@ -1832,10 +1948,18 @@ cudaError_t launch_lu_mixed(const Batch& bt, const float* A_hi, float* LU, int32
     SolveArgs g = a;
     g.bt.n_max = min(bt.n_max, kLargeM - 1);
     const size_t smem = lu_global_smem(g.bt.n_max);
-    e = ensure_smem(k_lu_global, smem);
-    if (e != cudaSuccess) return e;
-    k_lu_global<<<bt.B, kThreads, smem, s>>>(g);
-    e = cudaGetLastError();
+    auto go = [&](auto kernel) {
+      const cudaError_t r = ensure_smem(kernel, smem);
+      if (r != cudaSuccess) return r;
+      kernel<<<bt.B, kThreads, smem, s>>>(g);
+      return cudaGetLastError();
+    };
+    // three blocks per SM (80 registers, some spilled) where their shared memory fits
+    // and the batch fills them, else two with 128 registers (4096 x 256 panels 2566 us
+    // against 2781; 1216 x 400, whose panels leave room for two, 2510 against 2350; one
+    // of 300 238 against 207)
+    e = 3 * (smem + 1024) <= 228 * 1024 && bt.B > 2 * sm_count() ? go(k_lu_global<3>)
+                                                                 : go(k_lu_global<2>);
     if (e != cudaSuccess) return e;
   }
   return launch_gj_mixed(a, s);

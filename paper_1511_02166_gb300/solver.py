@@ -99,7 +99,7 @@ def lu_kind_by_size(count, m, sms):
     at most m unknowns on `sms` multiprocessors (1 through L2, 2 in shared memory)."""
     if m > LU_SMEM_MAX_M:
         return 1
-    return 2 if m <= 128 or count <= (2 if m <= 180 else 12) * sms else 1
+    return 2 if m <= 64 or (m > 160 and count <= sms) else 1
 
 
 def _require_cuda(device):

@@ -57,6 +57,34 @@ def test_lu_in_shared_memory_and_through_l2_agree(n):
     assert np.array_equal(out[0][1], out[1][1])
 
 
+@pytest.mark.parametrize("n", [31, 222, 223, 255, 256, 286, 351, 380, 384, 480, 639])
+def test_lu_through_l2_with_two_and_three_blocks_per_sm(n):
+    """The L2-resident LU's two forms (by batch and shared memory) do the same
+    operations; small batches are compared with the shared-memory form above."""
+    need_gpu()
+    import torch
+    from paper_1511_02166_gb300.solver import PanelBatch
+    base = _airfoils((n, max(3, n - 1)), seed=n)
+    one, many = base, inputs.pack([base.airfoil(b) for b in range(2)] * 160,
+                                  np.tile(base.alpha, 160))
+    out = []
+    for pop in (one, many):
+        pb = PanelBatch(pop.nodes, pop.offsets, pop.alpha, bucket_width=None)
+        pb.lu_kind = [1]
+        pb.run(with_grad=False)
+        assert int(pb.info.abs().max()) == 0
+        m = n + 1
+        A = (pb.A_hi[:m * m].double() + pb.A_lo[:m * m].double()).reshape(m, m)
+        x = torch.linalg.solve(A, pb.rhs[:m])
+        u = pb.u[:m].clone()
+        # the refinement stops at 1e-12 of the largest strength; the 64-bit solve's
+        # own error is cond(A) 2^-53 (up to ~1e4 here)
+        assert float((u - x).abs().max()) <= 1e-11 * float(x.abs().max())
+        out.append((pb.LU[:m * m].cpu().numpy().view(np.uint32), pb.piv[:m].cpu().numpy()))
+    assert np.array_equal(out[0][0], out[1][0])
+    assert np.array_equal(out[0][1], out[1][1])
+
+
 @pytest.mark.parametrize("sizes", [(3, 70), (65, 96, 97), (127, 128, 129), (160,), (255, 257, 31),
                                    (15, 16, 17, 400), (1030, 640)])
 @pytest.mark.parametrize("copies", [1, 40])
