@@ -44,6 +44,7 @@
 // exchanges, and the 32 x 32 diagonal blocks of L and U that follow the tiles
 // replaced by their inverses; the refinement (k_solve_mixed.cu) reads it in
 // that layout.
+#include <type_traits>
 #include <atomic>
 
 #include "tl_layout.cuh"
@@ -155,8 +156,10 @@ __global__ void __launch_bounds__(256, 3) k_large_diag(SolveArgs a, int K) {
   extern __shared__ __align__(16) unsigned char smraw[];
   float* D = reinterpret_cast<float*>(smraw);          // kBW x kLdD
   float* rows4 = D + kBW * kLdD;                       // 2 x 4 x 32: the warps' candidate rows
-  unsigned* red = reinterpret_cast<unsigned*>(rows4 + 256);  // 2 x 4 x 2: their keys, positions
-  int* sp = reinterpret_cast<int*>(red + 16);          // kBW
+  float* lt = rows4 + 256;                             // 32 x 32: the panel's L11 (tri_subst)
+  unsigned* red = reinterpret_cast<unsigned*>(lt + 1024);  // 2 x 4 x 2: keys, positions
+  float* rv = reinterpret_cast<float*>(red + 16);      // 2 x 4: the candidates' reciprocals
+  int* sp = reinterpret_cast<int*>(rv + 8);            // kBW
   const Batch& bt = a.bt;
   const int b = bt.order[blockIdx.x];
   int n, m;
@@ -172,9 +175,16 @@ __global__ void __launch_bounds__(256, 3) k_large_diag(SolveArgs a, int K) {
   auto dpos = [&](int r, int c) {
     return (K == 0) ? (int64_t)r * m + c : (int64_t)((c >> 5) << 12) + r * 32 + (c & 31);
   };
-  for (int e = tid; e < kBW * kBW; e += 256) {
-    const int r = e >> 7, c = e & 127;
-    D[r * kLdD + c] = (r < kb && c < kb) ? Td[dpos(r, c)] : 0.0f;
+  // 16 loads in flight per thread
+  for (int e0 = tid; e0 < kBW * kBW; e0 += 16 * 256) {
+    float v[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const int e = e0 + 256 * i, r = e >> 7, c = e & 127;
+      v[i] = (r < kb && c < kb) ? Td[dpos(r, c)] : 0.0f;
+    }
+#pragma unroll
+    for (int i = 0; i < 16; ++i) D[((e0 + 256 * i) >> 7) * kLdD + (e0 & 127)] = v[i];
   }
   __syncthreads();
   // Blocked in panels of 32 columns.  Per panel: warps 0-3 factor the panel
@@ -183,15 +193,19 @@ __global__ void __launch_bounds__(256, 3) k_large_diag(SolveArgs a, int K) {
   // threads and `pos` tracks their current position, so an exchange is
   // bookkeeping plus one sp entry.  Per column, one 128-thread barrier: each
   // warp finds its candidate (largest |x|, the lowest position among equal
-  // maxima) and puts its key, position and whole row in shared memory (two
+  // maxima) and puts its key, position, reciprocal and row in shared memory (two
   // buffers, alternating by column); after the barrier every thread picks the
-  // pivot among the four and reads its row; the rank-1 update in registers.  The step loop is rolled, the columns
-  // rotating through the registers (x[0] is the current one) so that every
-  // register index is a constant; each finished entry goes to the row's own
-  // place in D (by original row), and the rows are written back in their final
-  // order at the end.  Then the whole block applies the panel's exchanges to
-  // the other columns, solves U12 = L11^{-1} A12 (a thread per column) and
-  // updates the trailing block in 4 x 4 register tiles.
+  // pivot among the four and reads its row; the rank-1 update in registers.  The
+  // step loop is rolled, the columns rotating down the registers as they are
+  // updated (x[0] is the current one) so that every register index is a constant,
+  // in four groups of eight steps that narrow from 31 columns to 7; each finished
+  // entry goes to the row's own place in D (by original row), and the rows are
+  // written back in their final order at the end.  Every thread takes its entry's
+  // reciprocal while the pivot is searched: after the search it was a third of the
+  // step.  Then the whole block applies the panel's exchanges to the other columns,
+  // solves U12 = L11^{-1} A12 (a thread per column, tri_subst) and updates the
+  // trailing block, a warp 8 rows at a time with the columns across its lanes.
+  // The kernel is one chain per airfoil, 128 dependent steps a block.
   __shared__ int zero_pivot;
   if (tid == 0) zero_pivot = -1;
   __syncthreads();
@@ -206,68 +220,74 @@ __global__ void __launch_bounds__(256, 3) k_large_diag(SolveArgs a, int K) {
       int pos = tid;
       bool done = tid >= nrow;
       int fz = -1;
+      auto steps = [&](auto width) {
+        constexpr int W = decltype(width)::value;
 #pragma unroll 1
-      for (int q = 0; q < 32; ++q) {
-        const bool act = q < w && fz < 0;  // uniform over the 128 threads
-        const float v = (act && !done) ? fabsf(x[0]) : -1.0f;
-        const unsigned key = (v >= 0.0f) ? __float_as_uint(v) + 1u : 0u;
-        const unsigned wm = __reduce_max_sync(0xffffffffu, key);
-        const unsigned wp = __reduce_min_sync(0xffffffffu, key == wm ? (unsigned)pos : 0xffffu);
-        float* slot = rows4 + (q & 1) * 128;
-        unsigned* rk = red + (q & 1) * 8;
-        if (key == wm && pos == (int)wp) {  // the warp's candidate (one lane)
+        for (int lq = 0; lq < 8; ++lq) {
+          const int q = 32 - W + lq;
+          const bool act = q < w && fz < 0;  // uniform over the 128 threads
+          const float rc = __frcp_rn(x[0]);
+          asm volatile("" ::"f"(rc));  // here, not in the candidate's branch
+          const float v = (act && !done) ? fabsf(x[0]) : -1.0f;
+          const unsigned key = (v >= 0.0f) ? __float_as_uint(v) + 1u : 0u;
+          const unsigned wm = __reduce_max_sync(0xffffffffu, key);
+          const unsigned wp = __reduce_min_sync(0xffffffffu, key == wm ? (unsigned)pos : 0xffffu);
+          float* slot = rows4 + (q & 1) * 128;
+          unsigned* rk = red + (q & 1) * 8;
+          float* ri = rv + (q & 1) * 4;
+          if (key == wm && pos == (int)wp) {  // the warp's candidate (one lane)
 #pragma unroll
-          for (int t = 0; t < 32; t += 4)
-            *reinterpret_cast<float4*>(slot + warp * 32 + t) =
-                make_float4(x[t], x[t + 1], x[t + 2], x[t + 3]);
-        }
-        if (lane == 0) {
-          rk[warp] = wm;
-          rk[4 + warp] = wp;
-        }
-        asm volatile("bar.sync 1, 128;" ::: "memory");
-        unsigned mx = rk[0], pm = rk[4];
-        int ww = 0;
-#pragma unroll
-        for (int k = 1; k < 4; ++k) {
-          const unsigned kk = rk[k], pk = rk[4 + k];
-          if (kk > mx || (kk == mx && pk < pm)) {
-            mx = kk;
-            pm = pk;
-            ww = k;
+            for (int t = 0; t < W; t += 4)
+              *reinterpret_cast<float4*>(slot + warp * 32 + t) =
+                  make_float4(x[t], x[t + 1], x[t + 2], x[t + 3]);
+            ri[warp] = rc;
           }
-        }
-        const bool ok = act && mx > 1u;  // mx <= 1: exactly zero (or NaN) column
-        if (act && !ok) fz = q;
-        const bool piv = ok && key == mx && pos == (int)pm;
-        if (ok && tid == 0) sp[c0 + q] = c0 + (int)pm;
-        if (ok && pos == q && !piv) pos = (int)pm;
-        if (piv) {
-          pos = q;
-          done = true;
-        }
-        // the pivot row, four columns at a time straight into the update
-        const float* prow = slot + ww * 32;
-        const float4 f0 = *reinterpret_cast<const float4*>(prow);
-        const bool elim = ok && !done;
-        const float l = x[0] * __frcp_rn(f0.x);
-        const float le = elim ? l : 0.0f;
-        x[1] = fmaf(-le, f0.y, x[1]);
-        x[2] = fmaf(-le, f0.z, x[2]);
-        x[3] = fmaf(-le, f0.w, x[3]);
+          if (lane == 0) {
+            rk[warp] = wm;
+            rk[4 + warp] = wp;
+          }
+          asm volatile("bar.sync 1, 128;" ::: "memory");
+          unsigned mx = rk[0], pm = rk[4];
+          int ww = 0;
 #pragma unroll
-        for (int t = 4; t < 32; t += 4) {
-          const float4 r4 = *reinterpret_cast<const float4*>(prow + t);
-          x[t] = fmaf(-le, r4.x, x[t]);
-          x[t + 1] = fmaf(-le, r4.y, x[t + 1]);
-          x[t + 2] = fmaf(-le, r4.z, x[t + 2]);
-          x[t + 3] = fmaf(-le, r4.w, x[t + 3]);
-        }
-        if (tid < nrow && q < w) D[(c0 + tid) * kLdD + c0 + q] = elim ? l : x[0];
+          for (int k = 1; k < 4; ++k) {
+            const unsigned kk = rk[k], pk = rk[4 + k];
+            if (kk > mx || (kk == mx && pk < pm)) {
+              mx = kk;
+              pm = pk;
+              ww = k;
+            }
+          }
+          const bool ok = act && mx > 1u;  // mx <= 1: exactly zero (or NaN) column
+          if (act && !ok) fz = q;
+          const bool piv = ok && key == mx && pos == (int)pm;
+          if (ok && tid == 0) sp[c0 + q] = c0 + (int)pm;
+          if (ok && pos == q && !piv) pos = (int)pm;
+          if (piv) {
+            pos = q;
+            done = true;
+          }
+          const bool elim = ok && !done;
+          const float l = x[0] * ri[ww];
+          const float le = elim ? l : 0.0f;
+          if (tid < nrow && q < w) D[(c0 + tid) * kLdD + c0 + q] = elim ? l : x[0];
+          // the pivot row, four columns at a time straight into the update
+          const float* prow = slot + ww * 32;
 #pragma unroll
-        for (int t = 0; t < 31; ++t) x[t] = x[t + 1];
-        x[31] = 0.0f;
-      }
+          for (int t = 0; t < W; t += 4) {
+            const float4 r4 = *reinterpret_cast<const float4*>(prow + t);
+            if (t > 0) x[t - 1] = fmaf(-le, r4.x, x[t]);
+            x[t] = fmaf(-le, r4.y, x[t + 1]);
+            x[t + 1] = fmaf(-le, r4.z, x[t + 2]);
+            x[t + 2] = fmaf(-le, r4.w, x[t + 3]);
+          }
+          x[W - 1] = 0.0f;
+        }
+      };
+      steps(std::integral_constant<int, 32>{});
+      if (w > 8) steps(std::integral_constant<int, 24>{});
+      if (w > 16) steps(std::integral_constant<int, 16>{});
+      if (w > 24) steps(std::integral_constant<int, 8>{});
       if (fz >= 0 && tid == 0) zero_pivot = c0 + fz;
       asm volatile("bar.sync 1, 128;" ::: "memory");
       // the panel's rows in their final order
@@ -288,61 +308,76 @@ __global__ void __launch_bounds__(256, 3) k_large_diag(SolveArgs a, int K) {
       }
       return;
     }
-    // the panel's exchanges, in order, on the block's other columns
-    for (int c = tid; c < kb; c += 256) {
-      if (c >= c0 && c < c0 + w) continue;
-      for (int q = c0; q < c0 + w; ++q) {
-        const int p = sp[q];
-        if (p != q) {
-          const float t = D[q * kLdD + c];
-          D[q * kLdD + c] = D[p * kLdD + c];
-          D[p * kLdD + c] = t;
+    // the panel's exchanges, in order, on the block's other columns (each warp finds
+    // the rows that move by a vote)
+    const int sq = lane < w ? sp[c0 + lane] : 0;
+    const unsigned moves = __ballot_sync(0xffffffffu, lane < w && sq != c0 + lane);
+    if (moves)
+      for (int cw = 32 * warp; cw < kb; cw += 256) {
+        const int c = cw + lane;
+        for (unsigned left = moves; left; left &= left - 1) {
+          const int q = c0 + __ffs(left) - 1;
+          const int p = __shfl_sync(0xffffffffu, sq, q - c0);
+          if (c < kb && (c < c0 || c >= c0 + w)) {
+            const float t = D[q * kLdD + c];
+            D[q * kLdD + c] = D[p * kLdD + c];
+            D[p * kLdD + c] = t;
+          }
         }
       }
-    }
-    __syncthreads();
     const int c1 = c0 + w;
+    if (c1 < kb)  // L11 as tri_subst reads it (w == 32)
+      for (int e = tid; e < 1024; e += 256) {
+        const int q = e >> 5, r = q + 1 + (e & 31);
+        lt[e] = r < 32 ? D[(c0 + r) * kLdD + c0 + q] : 0.0f;
+      }
+    __syncthreads();
     if (c1 >= kb) break;
-    // U12 = L11^{-1} A12 on rows c0..c1-1, columns c1..kb-1 (unit lower L11;
-    // here w == 32): a thread per column in registers, right-looking
-    for (int c = c1 + tid; c < kb; c += 256) {
-      float col[32];
+    // U12 = L11^{-1} A12 on rows c0..c1-1, columns c1..kb-1 (unit lower L11)
+    if (c1 + tid < kb) {
+      float* col = D + c0 * kLdD + c1 + tid;
+      float x[32];
 #pragma unroll
-      for (int t = 0; t < 32; ++t) col[t] = D[(c0 + t) * kLdD + c];
-#pragma unroll
-      for (int q = 0; q < 32; ++q)
-#pragma unroll
-        for (int t = q + 1; t < 32; ++t) col[t] = fmaf(-D[(c0 + t) * kLdD + c0 + q], col[q], col[t]);
-#pragma unroll
-      for (int t = 1; t < 32; ++t) D[(c0 + t) * kLdD + c] = col[t];
+      for (int t = 0; t < 32; ++t) x[t] = col[t * kLdD];
+      tri_subst<false>(x, lt, nullptr, [&](int q, float v) { col[q * kLdD] = v; });
     }
     __syncthreads();
-    // trailing block: rows and columns c1..kb-1, D -= L21 U12, 4 x 4 per task
-    const int nr = kb - c1, nb4 = (nr + 3) >> 2;
-    for (int task = tid; task < nb4 * nb4; task += 256) {
-      const int r0 = c1 + 4 * (task / nb4), cc0 = c1 + 4 * (task % nb4);
-      float acc[4][4];
+    // trailing block: rows and columns c1..kb-1, D -= L21 U12, a warp 8 rows x 32 J
+    // columns at a time
+    const int nr = kb - c1;
+    auto update = [&](auto cols) {
+      constexpr int J = decltype(cols)::value;
+      for (int rt = warp; 8 * rt < nr; rt += 8) {
+        float* Dr = D + (c1 + 8 * rt) * kLdD;  // (rows beyond kb: zeros of the block)
+        float acc[8][J];
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) acc[i][jj] = 0.0f;
-      for (int t = 0; t < w; ++t) {
-        float av[4], bw[4];
+          for (int j = 0; j < J; ++j) acc[i][j] = 0.0f;
+#pragma unroll 4
+        for (int t = 0; t < 32; ++t) {
+          float bw[J];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) av[i] = (r0 + i < kb) ? D[(r0 + i) * kLdD + c0 + t] : 0.0f;
+          for (int j = 0; j < J; ++j) bw[j] = D[(c0 + t) * kLdD + c1 + lane + 32 * j];
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) bw[jj] = (cc0 + jj < kb) ? D[(c0 + t) * kLdD + cc0 + jj] : 0.0f;
+          for (int i = 0; i < 8; ++i) {
+            const float av = Dr[i * kLdD + c0 + t];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int j = 0; j < J; ++j) acc[i][j] = fmaf(av, bw[j], acc[i][j]);
+          }
+        }
 #pragma unroll
-          for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fmaf(av[i], bw[jj], acc[i][jj]);
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < J; ++j) Dr[i * kLdD + c1 + lane + 32 * j] -= acc[i][j];
       }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-          if (r0 + i < kb && cc0 + jj < kb) D[(r0 + i) * kLdD + cc0 + jj] -= acc[i][jj];
-    }
+    };
+    if (nr > 64)
+      update(std::integral_constant<int, 3>{});
+    else if (nr > 32)
+      update(std::integral_constant<int, 2>{});
+    else
+      update(std::integral_constant<int, 1>{});
     __syncthreads();
   }
   if (K >= 1) {
@@ -400,7 +435,9 @@ __global__ void __launch_bounds__(256, 3) k_large_diag(SolveArgs a, int K) {
   }
 }
 
-size_t large_diag_smem() { return (size_t)kBW * kLdD * 4 + 256 * 4 + 16 * 4 + 3 * kBW * 4; }
+size_t large_diag_smem() {
+  return (size_t)kBW * kLdD * 4 + (256 + 1024) * 4 + (16 + 8) * 4 + 3 * kBW * 4;
+}
 
 // U12 = L11^{-1} A12 and L21 = A21 U11^{-1} as products with the explicit
 // inverses of the two triangles of the factored diagonal block K.  Per block:

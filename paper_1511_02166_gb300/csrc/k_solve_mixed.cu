@@ -170,38 +170,9 @@ __device__ __forceinline__ void diag_tab_init(DiagTab& d) {
     if ((e & 31) >= 31 - (e >> 5)) d.u[e] = d.l[e] = 0.0f;
 }
 
-// Substitution against the table, right-looking, a right-hand side per thread in
-// x: SCALE, x <- x U^{-1} (a row); else x <- L^{-1} x (a column, unit L).  Each
-// final entry goes to out(q, value).  The entries rotate down the registers as
-// they are updated (x[0] is the current one), in four groups of eight steps
-// whose updates narrow from 31 to 7 entries: 608 multiply-adds a thread for the
-// 496 of the triangle, and a loop body short enough to stay in the instruction
-// cache (the fully unrolled form with one scalar load per multiply-add took
-// 8-12 thousand cycles a panel, bound by its shared-memory loads).
-template <int W, bool SCALE, class Out>
-__device__ __forceinline__ void tri_group(float (&x)[32], const DiagTab& d, const Out& out) {
-#pragma unroll 1
-  for (int lq = 0; lq < 8; ++lq) {
-    const int q = 32 - W + lq;
-    const float4* m = reinterpret_cast<const float4*>((SCALE ? d.u : d.l) + q * 32);
-    const float xq = SCALE ? x[0] * d.rinv[q] : x[0];
-    out(q, xq);
-#pragma unroll
-    for (int t4 = 0; t4 < W / 4; ++t4) {
-      const float4 f = m[t4];
-      x[4 * t4] = fmaf(-xq, f.x, x[4 * t4 + 1]);
-      x[4 * t4 + 1] = fmaf(-xq, f.y, x[4 * t4 + 2]);
-      x[4 * t4 + 2] = fmaf(-xq, f.z, x[4 * t4 + 3]);
-      x[4 * t4 + 3] = (4 * t4 + 4 < W) ? fmaf(-xq, f.w, x[(4 * t4 + 4) & 31]) : 0.0f;
-    }
-  }
-}
 template <bool SCALE, class Out>
 __device__ __forceinline__ void tri_subst(float (&x)[32], const DiagTab& d, const Out& out) {
-  tri_group<32, SCALE>(x, d, out);
-  tri_group<24, SCALE>(x, d, out);
-  tri_group<16, SCALE>(x, d, out);
-  tri_group<8, SCALE>(x, d, out);
+  tri_subst<SCALE>(x, SCALE ? d.u : d.l, d.rinv, out);
 }
 
 // ---------------------------------------------------------------------------
