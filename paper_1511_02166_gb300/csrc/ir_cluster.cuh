@@ -270,7 +270,8 @@ __device__ void cluster_residuals(cg::cluster_group& cl, const float* __restrict
   const int gw = rank * kIrClWarps + warp, GW = C * kIrClWarps;
   if (fw) {
     const float *xh = sm.xh[0], *xl = sm.xl[0];
-    RowSums<Acc, ClusterRhs, float> sums(ClusterRhs{R0, cl, C}, sm.r[0], gw, GW, m);
+    const ClusterRhs rhs{R0, cl, C};
+    RowSums<Acc, ClusterRhs, float> sums(rhs, sm.r[0], gw, GW, m);
     for (int j = gw; j < m; j += GW) {
       Acc acc;
       resacc_init(acc);

@@ -1341,6 +1341,8 @@ struct RowSums {
     for (int t = 0; t < 4; ++t) resacc_init(v[t]);
     resacc_init(keep);
   }
+  // b is kept by reference until finish(): a temporary would be gone by then
+  RowSums(const Rhs&&, RT*, int, int, int) = delete;
   __device__ __forceinline__ void add(const Acc& a) {
     if constexpr (!QUAD) {
       keep = sel_acc((int)(threadIdx.x & 31) == (i & 31), warp_sum_res(a), keep);
