@@ -267,6 +267,10 @@ int panel_viscous(int B, const double* nodes, const int64_t* node_offsets, const
  *   grad_cl [B] f64 upstream gradient (NULL means 1); grad_nodes [sum n_b][2]
  *   f64 output.  info [B] i32 (in/out): airfoils with info[b] != 0 are skipped
  *   (gradient set to NaN); the refinement of lambda may set PANEL_INFO_NOCONV.
+ *   Repeating a call on the same device gives the same bits in PANEL_MIXED mode
+ *   with n_max <= 256 (sums in a fixed order, which depends on the batch); above
+ *   it, and in PANEL_FP64 mode, the last bits of grad_nodes vary from run to run
+ *   (FP64 atomics).
  */
 int panel_adjoint(int B, int n_max, int flags, const double* nodes, const int64_t* node_offsets,
                   const int64_t* mat_offsets, const int32_t* order, const double* A64,
@@ -312,7 +316,8 @@ int panel_polar(int B, int n_max, int flags, const double* nodes, const int64_t*
  *   u [sum m_b] the solved strengths; w_cl [B] (NULL = 0); w_u [sum m_b] packed
  *   like u and w_cp [sum n_b] packed like the nodes (NULL = 0); lambda
  *   [sum m_b] f64 output;
- *   grad_nodes [sum n_b][2] f64 output (NaN where info[b] != 0).
+ *   grad_nodes [sum n_b][2] f64 output (NaN where info[b] != 0), repeated bit for
+ *   bit under the same conditions as panel_adjoint's.
  */
 int panel_vjp(int B, int n_max, int flags, const double* nodes, const int64_t* node_offsets,
               const int64_t* mat_offsets, const int32_t* order, const float* A_hi,

@@ -39,10 +39,13 @@
 // accumulate in the lane's registers (double-float; A_i = -S_i - B_i by
 // translation invariance), the row sums P_j are warp-reduced and kept as one
 // double-float partial per warp in shared memory, summed at the end
-// (n <= kPartialsN).  Larger airfoils and small batches take k_adjoint_df_split:
-// one block per (airfoil, 64 panels, range of rows), every term of the formula
-// above added into the caller's gradient buffer by FP64 atomics once per row
-// window, column or node (a few per pair row, not per pair).
+// (n <= kPartialsN).  Small batches of such airfoils take k_adjoint_df_cluster, a
+// cluster of blocks per airfoil; both sum in a fixed order.  Larger airfoils take
+// k_adjoint_df_split: one block per (airfoil, 64 panels, range of rows), every term
+// of the formula above added into the caller's gradient buffer by FP64 atomics once
+// per row window, column or node (a few per pair row, not per pair).
+#include <cooperative_groups.h>
+
 #include "panel_common.cuh"
 #include "panel_df.cuh"
 
@@ -205,14 +208,53 @@ __device__ __forceinline__ df2 warp_rowsum4(const df2 (&v)[4], int lane) {
   return k;
 }
 
-__device__ __forceinline__ df2 warp_sum_df2(df2 a) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    a = df_add(a, mkdf(__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)));
-  return a;
+// The rows [j0, j1) against the lane's panel ii (its strength ui, 0 where !ok; all
+// lanes of the warp call): S_i += lambda_j dG/dp and sum lambda_j K into the lane's
+// accumulators, and the row sums u_i dG/dp over the lanes to out(row, x, y), one lane
+// per row, four rows at a time: the terms of a window are shifted into rx/ry (static
+// register indices with a rolled loop) and reduced together.
+template <class Out>
+__device__ __forceinline__ void adjoint_rows(const float* pc, int ld, int ii, bool ok, df2 ui,
+                                             const float* lamh, const float* laml, int j0, int j1,
+                                             const float4* tlog, const float2* tatan, df2& sSx,
+                                             df2& sSy, df2& sKr, df2& sKi, const Out& out) {
+  const int lane = threadIdx.x & 31;
+  df2 rx[4], ry[4];
+  for (int w0 = j0; w0 < j1; w0 += 4) {
+#pragma unroll 1
+    for (int t = 0; t < 4; ++t) {
+      const int j = w0 + t;
+      df2 vx = mkdf(0.0f), vy = mkdf(0.0f);
+      if (j < j1) {
+        const point3 pj = load_point(pc, ld, j);
+        df2 gpx, gpy, kr, ki;
+        panel_dG_df(pj, pc, ld, ii, ii == j, tlog, tatan, gpx, gpy, kr, ki);
+        const df2 lj = mkdf(lamh[j], laml[j]);
+        // S_i += lambda_j gp, sum lambda_j K (B_i = R_t sum lambda K - S_i / 2)
+        acc_add_prod(sSx, lj, gpx);
+        acc_add_prod(sSy, lj, gpy);
+        acc_add_prod(sKr, lj, kr);
+        acc_add_prod(sKi, lj, ki);
+        if (ok) {
+          vx = df_mul(ui, gpx);
+          vy = df_mul(ui, gpy);
+        }
+      }
+      rx[0] = rx[1]; rx[1] = rx[2]; rx[2] = rx[3]; rx[3] = vx;
+      ry[0] = ry[1]; ry[1] = ry[2]; ry[2] = ry[3]; ry[3] = vy;
+    }
+    acc_norm(sSx);
+    acc_norm(sSy);
+    acc_norm(sKr);
+    acc_norm(sKi);
+    const df2 sx = warp_rowsum4(rx, lane), sy = warp_rowsum4(ry, lane);
+    const int jr = w0 + (lane >> 3);
+    if ((lane & 7) == 0 && jr < j1) out(jr, sx, sy);
+  }
 }
 
 constexpr int kPartialsN = 256;
+namespace cg = cooperative_groups;
 
 __global__ void __launch_bounds__(256) k_adjoint_df(
     Batch bt, const double* __restrict__ u, const double* __restrict__ lambda,
@@ -267,44 +309,12 @@ __global__ void __launch_bounds__(256) k_adjoint_df(
     const int ii = ok ? i : n - 1;
     const df2 ui = ok ? df_from_double(ub[ii]) : mkdf(0.0f);
     df2 sSx = mkdf(0.0f), sSy = mkdf(0.0f), sKr = mkdf(0.0f), sKi = mkdf(0.0f);
-    // rows in windows of 4: the lane's u_i dG/dp terms are shifted into rx/ry
-    // (static register indices with a rolled loop) and reduced per window
-    df2 rx[4], ry[4];
-    for (int j0 = 0; j0 < n; j0 += 4) {
-#pragma unroll 1
-      for (int t = 0; t < 4; ++t) {
-        const int j = j0 + t;
-        df2 vx = mkdf(0.0f), vy = mkdf(0.0f);
-        if (j < n) {
-          const point3 pj = load_point(pc, ld, j);
-          df2 gpx, gpy, kr, ki;
-          panel_dG_df(pj, pc, ld, ii, ii == j, tlog, tatan, gpx, gpy, kr, ki);
-          const df2 lj = mkdf(lamh[j], laml[j]);
-          // S_i += lambda_j gp, sum lambda_j K (B_i = R_t sum lambda K - S_i / 2)
-          acc_add_prod(sSx, lj, gpx);
-          acc_add_prod(sSy, lj, gpy);
-          acc_add_prod(sKr, lj, kr);
-          acc_add_prod(sKi, lj, ki);
-          if (ok) {
-            vx = df_mul(ui, gpx);
-            vy = df_mul(ui, gpy);
-          }
-        }
-        rx[0] = rx[1]; rx[1] = rx[2]; rx[2] = rx[3]; rx[3] = vx;
-        ry[0] = ry[1]; ry[1] = ry[2]; ry[2] = ry[3]; ry[3] = vy;
-      }
-      acc_norm(sSx);
-      acc_norm(sSy);
-      acc_norm(sKr);
-      acc_norm(sKi);
-      const df2 sx = warp_rowsum4(rx, lane), sy = warp_rowsum4(ry, lane);
-      const int jr = j0 + (lane >> 3);
-      if ((lane & 7) == 0 && jr < n) {
-        const float4 q = Pw[warp * ld + jr];
-        const df2 px = df_add(mkdf(q.x, q.y), sx), py = df_add(mkdf(q.z, q.w), sy);
-        Pw[warp * ld + jr] = make_float4(px.hi, px.lo, py.hi, py.lo);
-      }
-    }
+    adjoint_rows(pc, ld, ii, ok, ui, lamh, laml, 0, n, tlog, tatan, sSx, sSy, sKr, sKi,
+                 [&](int jr, const df2& sx, const df2& sy) {
+                   const float4 q = Pw[warp * ld + jr];
+                   const df2 px = df_add(mkdf(q.x, q.y), sx), py = df_add(mkdf(q.z, q.w), sy);
+                   Pw[warp * ld + jr] = make_float4(px.hi, px.lo, py.hi, py.lo);
+                 });
     if (ok) {
       // B_i = R_t K - S_i / 2 with the panel's FP64 unit tangent; A_i = -S_i - B_i
       const int i1 = (i + 1 == n) ? 0 : i + 1;
@@ -359,7 +369,175 @@ __global__ void __launch_bounds__(256) k_adjoint_df(
 }
 
 // ---------------------------------------------------------------------------
-// Large airfoils and small batches (adjoint_split): block (x, y, z) takes the
+// Small batches of airfoils of up to kPartialsN panels: the C blocks of a
+// cluster share one airfoil.  Block `rank` takes the rows (control points)
+// [rank per, rank per + per) against every panel; within the block a warp takes
+// 32 panels and, where there are fewer such groups than warps, a part of the rows.
+// Each block prepares the constants of the panels of its own rows (~120 FP64
+// operations a panel, on a pipe of 1/74 of the FP32 rate) and copies the others
+// from its neighbours.  Its row sums P are complete (all panels); its sums
+// over rows are partial, and the block that owns panel i's node adds the C
+// blocks' parts through distributed shared memory, in the order of the ranks.
+// Every sum is in a fixed order: the same batch gives the same bits in every run
+// (the blocks of k_adjoint_df_split, which add by FP64 atomics, do not).
+// ---------------------------------------------------------------------------
+template <int NT>
+__host__ __device__ constexpr size_t adjoint_cluster_smem(int n_max, int C) {
+  const size_t per = (size_t)(n_max + C - 1) / C;
+  return 257 * 16 + 34 * 8 + 8 * per * 16 + (size_t)NT * 32 + 6 * per * 8 + 6 * (per + 1) * 8 +
+         (size_t)n_max * 4 * 2 + (size_t)kPanelFields * n_max * 4;
+}
+
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_adjoint_df_cluster(
+    Batch bt, const double* __restrict__ u, const double* __restrict__ lambda,
+    const double* __restrict__ alpha, const double* __restrict__ vinf,
+    const double* __restrict__ chord, const double* __restrict__ grad_cl,
+    double* __restrict__ grad, const int32_t* __restrict__ info, int lam_weighted) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  cg::cluster_group cl = cg::this_cluster();
+  const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+  const int ld = bt.n_max, pmax = (ld + C - 1) / C;
+  float4* tlog = reinterpret_cast<float4*>(smraw);        // 257
+  float2* tatan = reinterpret_cast<float2*>(tlog + 257);  // 34
+  float4* Pw = reinterpret_cast<float4*>(tatan + 34);     // 8 x pmax: row sums by column group
+  float4* Sp = Pw + 8 * pmax;                             // 2 x NT: (S, K) by part and panel
+  double* P = reinterpret_cast<double*>(Sp + 2 * NT);     // 2 pmax
+  double* E = P + 2 * pmax;                               // 4 pmax: node_terms
+  double* T = E + 4 * pmax;                               // 6 (pmax + 1): P, A, B of a panel
+  float* lamh = reinterpret_cast<float*>(T + 6 * (pmax + 1));  // n_max
+  float* laml = lamh + ld;
+  float* pc = laml + ld;                                  // kPanelFields * n_max
+
+  const int b = bt.order[blockIdx.x / C];
+  const int n = airfoil_n(bt, b);
+  double* gout = grad + 2 * bt.node_off[b];
+  const int tid = threadIdx.x;
+  if ((info && info[b] != 0) || n > ld || n < 3) {  // the whole cluster
+    for (int k = rank * NT + tid; k < 2 * n; k += C * NT) gout[k] = nan("");
+    return;
+  }
+  const double* nodes = bt.nodes + 2 * bt.node_off[b];
+  const double* ub = u + vec_off(bt, b);
+  const double* lb = lambda + vec_off(bt, b);
+  const int per = (n + C - 1) / C;
+  const int jbeg = min(n, rank * per), jend = min(n, jbeg + per), nr = jend - jbeg;
+  df_stage_tables(tlog, tatan);
+  for (int k = jbeg + tid; k < jend; k += NT) {
+    const int k1 = (k + 1 == n) ? 0 : k + 1;
+    panel_constants(pc, ld, k, nodes[2 * k], nodes[2 * k + 1], nodes[2 * k1], nodes[2 * k1 + 1]);
+    const df2 l = df_from_double(lb[k]);
+    lamh[k] = l.hi;
+    laml[k] = l.lo;
+  }
+  cl.sync();
+  // the other blocks' constants
+  for (int k = tid; k < n; k += NT) {
+    const int r = k / per;
+    if (r == rank) continue;
+    const float* src = cl.map_shared_rank(pc, r) + k;
+#pragma unroll
+    for (int f = 0; f < kPanelFields; ++f) pc[f * ld + k] = src[f * ld];
+  }
+  __syncthreads();
+
+  const int lane = tid & 31, warp = tid >> 5;
+  const int ncb = (n + 31) >> 5, parts = max(1, NT / 32 / ncb);
+  const int cb = warp % ncb, part = warp / ncb;
+  if (warp == NT / 32 - 1) {
+    // what the end needs besides the sums, beside the other warps' rows: its square
+    // roots, divisions, sine and cosine are chains of FP64 operations
+    const double v = vinf ? vinf[b] : 1.0, c = chord ? chord[b] : 1.0;
+    for (int t = lane; t < nr; t += 32)
+      node_terms(nodes, ub, lb, n, jbeg + t, v, c, alpha[b], E[4 * t], E[4 * t + 1], E[4 * t + 2],
+                 E[4 * t + 3]);
+    for (int t = lane; t <= nr; t += 32) {  // the FP64 unit tangents
+      const int q = (jbeg + t == 0) ? n - 1 : jbeg + t - 1, q1 = (q + 1 == n) ? 0 : q + 1;
+      const double hx = nodes[2 * q1] - nodes[2 * q], hy = nodes[2 * q1 + 1] - nodes[2 * q + 1];
+      const double L = sqrt(hx * hx + hy * hy);
+      T[6 * t + 4] = hx / L;
+      T[6 * t + 5] = hy / L;
+    }
+  }
+  if (part < parts) {
+    const int i = cb * 32 + lane;
+    const bool ok = i < n;
+    const int ii = ok ? i : n - 1;
+    const df2 ui = ok ? df_from_double(ub[ii]) : mkdf(0.0f);
+    df2 sSx = mkdf(0.0f), sSy = mkdf(0.0f), sKr = mkdf(0.0f), sKi = mkdf(0.0f);
+    // whole windows of 4 rows
+    const int nwin = (nr + 3) >> 2;
+    const int j0 = jbeg + 4 * (nwin * part / parts);
+    const int j1 = min(jend, jbeg + 4 * (nwin * (part + 1) / parts));
+    adjoint_rows(pc, ld, ii, ok, ui, lamh, laml, j0, j1, tlog, tatan, sSx, sSy, sKr, sKi,
+                 [&](int jr, const df2& sx, const df2& sy) {
+                   Pw[cb * pmax + jr - jbeg] = make_float4(sx.hi, sx.lo, sy.hi, sy.lo);
+                 });
+    Sp[2 * tid] = make_float4(sSx.hi, sSx.lo, sSy.hi, sSy.lo);
+    Sp[2 * tid + 1] = make_float4(sKr.hi, sKr.lo, sKi.hi, sKi.lo);
+  }
+  __syncthreads();
+  auto add4 = [](float4& a, const float4& q) {
+    const df2 x = df_add(mkdf(a.x, a.y), mkdf(q.x, q.y)), y = df_add(mkdf(a.z, a.w), mkdf(q.z, q.w));
+    a = make_float4(x.hi, x.lo, y.hi, y.lo);
+  };
+  // the parts of panel `tid`, into part 0's place; the column groups of row `tid`
+  if (tid < n && parts > 1) {
+    float4 s = Sp[2 * tid], k = Sp[2 * tid + 1];
+    for (int p = 1; p < parts; ++p) {
+      add4(s, Sp[2 * (tid + 32 * ncb * p)]);
+      add4(k, Sp[2 * (tid + 32 * ncb * p) + 1]);
+    }
+    Sp[2 * tid] = s;
+    Sp[2 * tid + 1] = k;
+  }
+  for (int r = tid; r < nr; r += NT) {
+    float4 s = Pw[r];
+    for (int q = 1; q < ncb; ++q) add4(s, Pw[q * pmax + r]);
+    P[2 * r] = df_to_double(mkdf(s.x, s.y));
+    P[2 * r + 1] = df_to_double(mkdf(s.z, s.w));
+  }
+  cl.sync();
+  // the sums of the panels jbeg - 1 .. jend - 1, whose ends are the block's nodes
+  for (int t = tid; t <= nr && nr > 0; t += NT) {
+    const int q = (jbeg + t == 0) ? n - 1 : jbeg + t - 1;
+    float4 s = cl.map_shared_rank(Sp, 0)[2 * q], k = cl.map_shared_rank(Sp, 0)[2 * q + 1];
+    for (int r = 1; r < C; ++r) {
+      add4(s, cl.map_shared_rank(Sp, r)[2 * q]);
+      add4(k, cl.map_shared_rank(Sp, r)[2 * q + 1]);
+    }
+    const double* Pq = cl.map_shared_rank(P, q / per) + 2 * (q % per);
+    // B_i = R_t K - S_i / 2 with the panel's unit tangent; A_i = -S_i - B_i
+    double* o = T + 6 * t;
+    const double tx = o[4], ty = o[5];
+    const double Sx = df_to_double(mkdf(s.x, s.y)), Sy = df_to_double(mkdf(s.z, s.w));
+    const double Kr = df_to_double(mkdf(k.x, k.y)), Ki = df_to_double(mkdf(k.z, k.w));
+    const double bx = tx * Kr - ty * Ki - 0.5 * Sx, by = ty * Kr + tx * Ki - 0.5 * Sy;
+    o[0] = Pq[0];
+    o[1] = Pq[1];
+    o[2] = -(Sx + bx);
+    o[3] = -(Sy + by);
+    o[4] = bx;
+    o[5] = by;
+  }
+  cl.sync();  // (a barrier of the block; and no block leaves while others read it)
+  // se scales the explicit dCl/dx term, sl the lambda terms (as in k_adjoint_df)
+  const double se = grad_cl ? grad_cl[b] : (lam_weighted ? 0.0 : 1.0);
+  const double sl = lam_weighted ? 1.0 : se;
+  for (int t = tid; t < nr; t += NT) {
+    const int k = jbeg + t, km = (k == 0) ? n - 1 : k - 1;
+    const double *m = T + 6 * t, *o = m + 6;  // panels k - 1 and k
+    const double ex = E[4 * t], ey = E[4 * t + 1];
+    double gx = E[4 * t + 2], gy = E[4 * t + 3];
+    gx += kInvTwoPi * (0.5 * (lb[km] * m[0] + lb[k] * o[0]) + ub[k] * o[2] + ub[km] * m[4]);
+    gy += kInvTwoPi * (0.5 * (lb[km] * m[1] + lb[k] * o[1]) + ub[k] * o[3] + ub[km] * m[5]);
+    gout[2 * k] = se * ex + sl * gx;
+    gout[2 * k + 1] = se * ey + sl * gy;
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Large airfoils (more than kPartialsN panels): block (x, y, z) takes the
 // panels [C y, C y + C) of airfoil order[x], C = blockDim.x -- one 32-column
 // block per warp -- against the control points [R z, R z + R), R a multiple of
 // 4.  Shared memory holds the constants of the block's own panels and a window
@@ -401,16 +579,8 @@ __global__ void __launch_bounds__(256) k_adjoint_prepare(
   // se scales the explicit dCl/dx term, sl the lambda terms (as in k_adjoint_df)
   const double se = grad_cl ? grad_cl[b] : (lam_weighted ? 0.0 : 1.0);
   const double sl = lam_weighted ? 1.0 : se;
-  const double ca = cos(alpha[b]), sa = sin(alpha[b]);
-  const int km = (k == 0) ? n - 1 : k - 1;
-  const int k1 = (k + 1 == n) ? 0 : k + 1;
-  const double hkx = nodes[2 * k1] - nodes[2 * k], hky = nodes[2 * k1 + 1] - nodes[2 * k + 1];
-  const double hmx = nodes[2 * k] - nodes[2 * km], hmy = nodes[2 * k + 1] - nodes[2 * km + 1];
-  const double Lk = sqrt(hkx * hkx + hky * hky), Lm = sqrt(hmx * hmx + hmy * hmy);
-  const double ex = 2.0 / (v * c) * (ub[km] * hmx / Lm - ub[k] * hkx / Lk);
-  const double ey = 2.0 / (v * c) * (ub[km] * hmy / Lm - ub[k] * hky / Lk);
-  const double bx = 0.5 * v * (-sa) * (lb[km] + lb[k]);
-  const double by = 0.5 * v * ca * (lb[km] + lb[k]);
+  double ex, ey, bx, by;
+  node_terms(nodes, ub, lb, n, k, v, c, alpha[b], ex, ey, bx, by);
   gout[2 * k] = se * ex + sl * bx;
   gout[2 * k + 1] = se * ey + sl * by;
 }
@@ -574,12 +744,40 @@ static int split_rows(int B, int n_max) {
   return max(4, (int)((((n_max + z - 1) / z) + 3) & ~3ll));
 }
 
-// Up to kPartialsN panels a block per airfoil is the faster form once the
-// airfoils' 32-column warps fill eight warps on every SM (200 panels, us: 64
-// airfoils 239 against 138 split, 152: 238 / 246, 608: 611 / 742); below it the
-// split fills the chip (100 panels: 64 airfoils 145 -> 68, 304: 170 / 172).
-static bool adjoint_split(int B, int n_max) {
-  return n_max > kPartialsN || (long long)B * ((n_max + 31) / 32) < 8ll * sm_count();
+// A launch of k_adjoint_df_cluster: C blocks of nt threads per airfoil.
+struct AdjointCluster {
+  int C, nt;
+};
+template <class Go>
+static cudaError_t with_adjoint_cluster(int nt, const Go& go) {
+  return nt == 512 ? go(k_adjoint_df_cluster<512, 1>, adjoint_cluster_smem<512>)
+                   : go(k_adjoint_df_cluster<256, 3>, adjoint_cluster_smem<256>);
+}
+
+// The form of k_adjoint_df_cluster for B airfoils, or C = 0 for one block of
+// k_adjoint_df each, which is the faster form once the airfoils' 32-column warps
+// fill eight warps on every SM (200 panels, us: 608 airfoils 611 against 742 by
+// k_adjoint_df_split; 152 233 against 178 here).  A row costs a warp 1.5 us, a chain of
+// dependent operations, so below it the airfoil is cut into as many warps as run at
+// once: the first of these forms whose clusters are all resident (measured on 152
+// SMs, us, 200 panels; k_adjoint_df_split, whose atomics this replaces, behind the bar):
+//   16 x 512  1 airfoil 32 | 27, 7 32 | 47  8 x 512  12 42 | 53    16 x 256  20 57 | 65
+//   4 x 512   30 66 | 82                    8 x 256  38 90 | 90    2 x 512  76 108 | 126
+//   4 x 256   100 155 | 170                 1 x 512  152 178 | 223
+// and for fewer panels 2 x 256 (200 of 100 panels 103 | 134), 1 x 256 (304 of 64 68 | 91).
+static AdjointCluster adjoint_cluster(int B, int n_max) {
+  if (n_max > kPartialsN || (long long)B * ((n_max + 31) / 32) >= 8ll * sm_count()) return {0, 0};
+  constexpr AdjointCluster forms[] = {{16, 512}, {8, 512}, {16, 256}, {4, 512}, {8, 256},
+                                      {2, 512},  {4, 256}, {1, 512},  {2, 256}};
+  for (const AdjointCluster& f : forms) {
+    int fit = 0;
+    with_adjoint_cluster(f.nt, [&](auto kernel, auto smem) {
+      fit = cluster_capacity(kernel, f.C, f.nt, smem(kPartialsN, f.C));
+      return cudaSuccess;
+    });
+    if (B <= fit) return f;
+  }
+  return {1, 256};
 }
 
 size_t adjoint_df_smem(int n_max) {
@@ -603,13 +801,7 @@ cudaError_t launch_adjoint_df(const Batch& bt, const double* u, const double* la
                               const double* grad_cl, double* grad, const int32_t* info,
                               cudaStream_t s, bool lam_weighted) {
   cudaError_t e;
-  if (!adjoint_split(bt.B, bt.n_max)) {
-    const size_t smem = adjoint_df_smem(bt.n_max);
-    e = ensure_smem(k_adjoint_df, smem);
-    if (e != cudaSuccess) return e;
-    k_adjoint_df<<<bt.B, 256, smem, s>>>(bt, u, lambda, alpha, vinf, chord, grad_cl, grad, info,
-                                         lam_weighted ? 1 : 0);
-  } else {
+  if (bt.n_max > kPartialsN) {
     const int rows = split_rows(bt.B, bt.n_max);
     const size_t smem = adjoint_split_smem();
     e = ensure_smem(k_adjoint_df_split, smem);
@@ -620,7 +812,24 @@ cudaError_t launch_adjoint_df(const Batch& bt, const double* u, const double* la
     const dim3 grid(bt.B, (bt.n_max + kSplitCols - 1) / kSplitCols, (bt.n_max + rows - 1) / rows);
     k_adjoint_df_split<<<grid, kSplitCols, smem, s>>>(bt, u, lambda, grad_cl, grad, info,
                                                       lam_weighted ? 1 : 0, rows);
+    return cudaGetLastError();
   }
+  if (const AdjointCluster f = adjoint_cluster(bt.B, bt.n_max); f.C > 0)
+    return with_adjoint_cluster(f.nt, [&](auto kernel, auto smem_of) {
+      const size_t smem = smem_of(bt.n_max, f.C);
+      const cudaError_t r = ensure_smem(kernel, smem);
+      if (r != cudaSuccess) return r;
+      cudaLaunchAttribute at;
+      const cudaLaunchConfig_t cfg =
+          cluster_config(dim3(bt.B * f.C), dim3(f.C), f.nt, smem, s, &at);
+      return cudaLaunchKernelEx(&cfg, kernel, bt, u, lambda, alpha, vinf, chord, grad_cl, grad,
+                                info, lam_weighted ? 1 : 0);
+    });
+  const size_t smem = adjoint_df_smem(bt.n_max);
+  e = ensure_smem(k_adjoint_df, smem);
+  if (e != cudaSuccess) return e;
+  k_adjoint_df<<<bt.B, 256, smem, s>>>(bt, u, lambda, alpha, vinf, chord, grad_cl, grad, info,
+                                       lam_weighted ? 1 : 0);
   return cudaGetLastError();
 }
 

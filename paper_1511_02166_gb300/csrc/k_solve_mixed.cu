@@ -1672,7 +1672,7 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
       (reinterpret_cast<uintptr_t>(t32 + 32) + 15) & ~(uintptr_t)15);
   // The corrections: the forward one in y, the transposed one in z, which is
   // the transposed system's float copy of lambda (rewritten from lambda before
-  // it is read again); the transposed sweeps' 32-float group scratch is `red`
+  // it is read again); the transposed sweeps' 64-float group scratch is `red`
   // (free while the sweeps run).
   float* z = sys[1].xh;
   float* t32z = reinterpret_cast<float*>(red);
@@ -1964,41 +1964,9 @@ static cudaError_t launch_ir_shape(const SolveArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-static cudaLaunchConfig_t ir_cluster_config(int B, int n_max, int C, cudaStream_t s,
-                                            cudaLaunchAttribute* at) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(B * C);
-  cfg.blockDim = dim3(kIrClThreads);
-  cfg.dynamicSmemBytes = ir_cluster_smem(n_max);
-  cfg.stream = s;
-  at->id = cudaLaunchAttributeClusterDimension;
-  at->val.clusterDim.x = C;
-  at->val.clusterDim.y = at->val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cfg;
-}
-
-// Clusters of C blocks of k_ir_cluster the device holds at once (asked once per
-// device, for the largest airfoil; 0 if the query fails).
+// Clusters of C blocks of k_ir_cluster the device holds at once, of the largest airfoil.
 static int ir_cluster_capacity(int C) {
-  static std::mutex mu;
-  static std::map<std::pair<int, int>, int> known;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  std::lock_guard<std::mutex> lock(mu);
-  const auto it = known.find(std::make_pair(dev, C));
-  if (it != known.end()) return it->second;
-  int n = 0;
-  cudaLaunchAttribute at;
-  const cudaLaunchConfig_t cfg = ir_cluster_config(1, PANEL_N_MAX, C, nullptr, &at);
-  if (ensure_smem(k_ir_cluster, cfg.dynamicSmemBytes) != cudaSuccess ||
-      cudaOccupancyMaxActiveClusters(&n, k_ir_cluster, &cfg) != cudaSuccess) {
-    (void)cudaGetLastError();
-    n = 0;
-  }
-  known[std::make_pair(dev, C)] = n;
-  return n;
+  return cluster_capacity(k_ir_cluster, C, kIrClThreads, ir_cluster_smem(PANEL_N_MAX));
 }
 
 // Blocks per airfoil of a refinement by clusters, or 0 for k_ir_mixed: the most that
@@ -2019,7 +1987,8 @@ static int ir_cluster_blocks(const SolveArgs& a) {
 
 static cudaError_t launch_ir_cluster(const SolveArgs& a, int C, cudaStream_t s) {
   cudaLaunchAttribute at;
-  const cudaLaunchConfig_t cfg = ir_cluster_config(a.bt.B, a.bt.n_max, C, s, &at);
+  const cudaLaunchConfig_t cfg = cluster_config(dim3(a.bt.B * C), dim3(C), kIrClThreads,
+                                                ir_cluster_smem(a.bt.n_max), s, &at);
   return cudaLaunchKernelEx(&cfg, k_ir_cluster, a);
 }
 

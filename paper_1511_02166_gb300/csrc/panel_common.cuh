@@ -10,6 +10,7 @@
 
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <utility>
 
 #include "../../include/panel.h"
@@ -117,6 +118,25 @@ __device__ __forceinline__ int load_and_check_geometry(const double* nodes, int 
   return 0;
 }
 
+// The terms of dCl/dx_k that need no pair sums: the explicit one,
+// (2/(v c)) (gamma_{k-1} t_{k-1} - gamma_k t_k), and that of the right-hand side,
+// v/2 (-sin a, cos a) (lambda_{k-1} + lambda_k).
+__device__ __forceinline__ void node_terms(const double* nodes, const double* u,
+                                           const double* lambda, int n, int k, double v, double c,
+                                           double alpha, double& ex, double& ey, double& bx,
+                                           double& by) {
+  const double ca = cos(alpha), sa = sin(alpha);
+  const int km = (k == 0) ? n - 1 : k - 1;
+  const int k1 = (k + 1 == n) ? 0 : k + 1;
+  const double hkx = nodes[2 * k1] - nodes[2 * k], hky = nodes[2 * k1 + 1] - nodes[2 * k + 1];
+  const double hmx = nodes[2 * k] - nodes[2 * km], hmy = nodes[2 * k + 1] - nodes[2 * km + 1];
+  const double Lk = sqrt(hkx * hkx + hky * hky), Lm = sqrt(hmx * hmx + hmy * hmy);
+  ex = 2.0 / (v * c) * (u[km] * hmx / Lm - u[k] * hkx / Lk);
+  ey = 2.0 / (v * c) * (u[km] * hmy / Lm - u[k] * hky / Lk);
+  bx = 0.5 * v * (-sa) * (lambda[km] + lambda[k]);
+  by = 0.5 * v * ca * (lambda[km] + lambda[k]);
+}
+
 // Raise a kernel's dynamic shared-memory limit only when a launch needs more
 // than any earlier one on the current device: after a warm-up call no
 // attribute is set any more, so later calls can be captured into CUDA graphs.
@@ -138,6 +158,52 @@ inline cudaError_t ensure_smem_impl(const void* kernel, size_t bytes) {
 template <typename K>
 inline cudaError_t ensure_smem(K kernel, size_t bytes) {
   return ensure_smem_impl(reinterpret_cast<const void*>(kernel), bytes);
+}
+
+// Launch configuration of clusters of cluster.x x cluster.y blocks.
+inline cudaLaunchConfig_t cluster_config(dim3 grid, dim3 cluster, int threads, size_t smem,
+                                         cudaStream_t s, cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = cluster.x;
+  at->val.clusterDim.y = cluster.y;
+  at->val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
+// Clusters of C blocks of a kernel that the current device holds at once (asked once
+// per device; 0 if it cannot run them).  Sizes above 8 are allowed on the way.
+inline int cluster_capacity_impl(const void* kernel, int C, int threads, size_t smem) {
+  static std::mutex mu;
+  static std::map<std::tuple<int, const void*, int>, int> known;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  std::lock_guard<std::mutex> lock(mu);
+  const auto key = std::make_tuple(dev, kernel, C);
+  const auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  int n = 0;
+  cudaLaunchAttribute at;
+  const cudaLaunchConfig_t cfg = cluster_config(dim3(C), dim3(C), threads, smem, nullptr, &at);
+  if (ensure_smem_impl(kernel, smem) != cudaSuccess ||
+      (C > 8 && cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
+                    cudaSuccess) ||
+      cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+    (void)cudaGetLastError();
+    n = 0;
+  }
+  known[key] = n;
+  return n;
+}
+template <typename K>
+inline int cluster_capacity(K kernel, int C, int threads, size_t smem) {
+  return cluster_capacity_impl(reinterpret_cast<const void*>(kernel), C, threads, smem);
 }
 
 // Streaming multiprocessors of the current device (queried once per device;
