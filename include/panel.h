@@ -267,10 +267,10 @@ int panel_viscous(int B, const double* nodes, const int64_t* node_offsets, const
  *   grad_cl [B] f64 upstream gradient (NULL means 1); grad_nodes [sum n_b][2]
  *   f64 output.  info [B] i32 (in/out): airfoils with info[b] != 0 are skipped
  *   (gradient set to NaN); the refinement of lambda may set PANEL_INFO_NOCONV.
- *   Repeating a call on the same device gives the same bits in PANEL_MIXED mode
- *   with n_max <= 256 (sums in a fixed order, which depends on the batch); above
- *   it, and in PANEL_FP64 mode, the last bits of grad_nodes vary from run to run
- *   (FP64 atomics).
+ *   Repeating a call on the same device gives the same bits with n_max <= 256 in
+ *   PANEL_MIXED and n_max <= 64 in PANEL_FP64 mode (sums in a fixed order, which
+ *   depends on the batch); above that the last bits of grad_nodes vary from run
+ *   to run (FP64 atomics).
  */
 int panel_adjoint(int B, int n_max, int flags, const double* nodes, const int64_t* node_offsets,
                   const int64_t* mat_offsets, const int32_t* order, const double* A64,

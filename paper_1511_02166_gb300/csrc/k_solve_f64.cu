@@ -14,6 +14,8 @@
 // (100 panels: 436 us as four barriers a step on the matrix in L2).  The
 // substitutions, one warp per system with its vector in shared memory, multiply by
 // the reciprocals of U's diagonal formed beforehand.
+#include <cooperative_groups.h>
+
 #include "panel_common.cuh"
 
 namespace panel {
@@ -308,9 +310,12 @@ __global__ void __launch_bounds__(128) k_lambda_f64(Batch bt, const double* __re
 // of its panels, so that a small batch still uses every SM's FP64 pipe, the bound
 // here; a warp takes 31 panels (lane l the distance to node i0 + l: neighbouring
 // panels share its logarithm) and windows of four rows, whose sums over the lanes
-// take 6 additions instead of 20.  k_adjoint_prepare writes the terms without pair
-// sums first; everything else goes in by FP64 atomics, so the last bits vary between
-// runs.
+// take 6 additions instead of 20.  Above kFixedF64N panels k_adjoint_prepare writes the
+// terms without pair sums first and everything else goes in by FP64 atomics, so the
+// last bits vary between runs.  Up to kFixedF64N panels (FIXED) the row ranges of an
+// airfoil are a cluster: each block keeps its sums by warp, and the block that owns a
+// node adds them up through distributed shared memory, all in a fixed order.
+constexpr int kFixedF64N = 64;  // at most 6 blocks of 12 rows, 3 column blocks
 constexpr int kAdjF64Threads = 256;
 
 __device__ __forceinline__ double rowsum4_f64(const double (&v)[4], int lane) {
@@ -325,22 +330,34 @@ __device__ __forceinline__ double rowsum4_f64(const double (&v)[4], int lane) {
   return k + __shfl_xor_sync(0xffffffffu, k, 1);
 }
 
+template <bool FIXED>
 __global__ void __launch_bounds__(kAdjF64Threads) k_adjoint_f64(
     Batch bt, const double* __restrict__ u, const double* __restrict__ lambda,
-    const double* __restrict__ grad_cl, double* __restrict__ grad,
-    const int32_t* __restrict__ info, int rows) {
+    const double* __restrict__ alpha, const double* __restrict__ vinf,
+    const double* __restrict__ chord, const double* __restrict__ grad_cl,
+    double* __restrict__ grad, const int32_t* __restrict__ info, int rows) {
   extern __shared__ double sm[];  // the rows' control points, lambda, and P: 5 x rows
   const int b = bt.order[blockIdx.x];
   const int n = airfoil_n(bt, b);
   const int j0 = blockIdx.y * rows;
-  if ((info && info[b] != 0) || n > bt.n_max || n < 3 || j0 >= n) return;
-  const int nr = min(rows, n - j0);
+  double* gout = grad + 2 * bt.node_off[b];
+  if ((info && info[b] != 0) || n > bt.n_max || n < 3) {  // (the whole cluster)
+    if (FIXED)
+      for (int k = blockIdx.y * kAdjF64Threads + threadIdx.x; k < 2 * n;
+           k += gridDim.y * kAdjF64Threads)
+        gout[k] = nan("");
+    return;
+  }
+  if (!FIXED && j0 >= n) return;
+  const int nr = max(0, min(rows, n - j0));
   double *px = sm, *py = sm + rows, *lam = sm + 2 * rows, *P = sm + 3 * rows;
+  double* Pc = sm + 5 * rows;   // FIXED: P by column block, 3 x 2 rows
+  double* T = Pc + 6 * rows;    // FIXED: 6 (rows + 1): P, A, B of a panel
+  double* Cs = T + 6 * (rows + 1);  // FIXED: S, B by part and panel, 8 x 32 x 4
   const double* nodes = bt.nodes + 2 * bt.node_off[b];
   const double* ub = u + vec_off(bt, b);
   const double* lb = lambda + vec_off(bt, b);
-  double* gout = grad + 2 * bt.node_off[b];
-  const double w2pi = (grad_cl ? grad_cl[b] : 1.0) * kInvTwoPi;
+  const double gscale = grad_cl ? grad_cl[b] : 1.0, w2pi = gscale * kInvTwoPi;
   for (int k = threadIdx.x; k < nr; k += kAdjF64Threads) {
     const int j = j0 + k, j1 = (j + 1 == n) ? 0 : j + 1;
     px[k] = 0.5 * (nodes[2 * j] + nodes[2 * j1]);
@@ -392,11 +409,23 @@ __global__ void __launch_bounds__(kAdjF64Threads) k_adjoint_f64(
       const double sx = rowsum4_f64(vx, lane), sy = rowsum4_f64(vy, lane);
       const int r = w0 + (lane >> 3);
       if ((lane & 7) == 0 && r < r1) {
-        atomicAdd(&P[2 * r], sx);
-        atomicAdd(&P[2 * r + 1], sy);
+        if (FIXED) {
+          double* q = Pc + 2 * ((t % ncb) * rows + r);
+          q[0] = sx;
+          q[1] = sy;
+        } else {
+          atomicAdd(&P[2 * r], sx);
+          atomicAdd(&P[2 * r + 1], sy);
+        }
       }
     }
-    if (ok) {
+    if (FIXED) {
+      double* q = Cs + 4 * (32 * t + lane);
+      q[0] = Sx;
+      q[1] = Sy;
+      q[2] = Bx;
+      q[3] = By;
+    } else if (ok) {
       // u_i A_i belongs to node i (start of panel i), u_i B_i to node i + 1;
       // A_i = -S_i - B_i
       const double f = w2pi * ui;
@@ -407,14 +436,58 @@ __global__ void __launch_bounds__(kAdjF64Threads) k_adjoint_f64(
     }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < nr; k += kAdjF64Threads) {
-    // lambda_j P_j / 2 belongs to the nodes j and j + 1 (the ends of panel j)
-    const int j = j0 + k, j1 = (j + 1 == n) ? 0 : j + 1;
-    const double f = 0.5 * w2pi * lam[k];
-    atomicAdd(&gout[2 * j], f * P[2 * k]);
-    atomicAdd(&gout[2 * j + 1], f * P[2 * k + 1]);
-    atomicAdd(&gout[2 * j1], f * P[2 * k]);
-    atomicAdd(&gout[2 * j1 + 1], f * P[2 * k + 1]);
+  if constexpr (FIXED) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int nz = gridDim.y, tid = threadIdx.x;
+    // the column blocks of row `tid`; the parts of panel `tid`, into part 0's place
+    if (tid < 2 * nr) {
+      double v = Pc[tid];
+      for (int q = 1; q < ncb; ++q) v += Pc[2 * q * rows + tid];
+      P[tid] = v;
+    }
+    for (int e = tid; e < 4 * 32 * ncb; e += kAdjF64Threads)
+      for (int q = 1; q < parts; ++q) Cs[e] += Cs[4 * 32 * ncb * q + e];
+    cl.sync();
+    // the sums of the panels j0 - 1 .. j0 + nr - 1, whose ends are the block's nodes
+    for (int t = tid; t <= nr && nr > 0; t += kAdjF64Threads) {
+      const int q = (j0 + t == 0) ? n - 1 : j0 + t - 1, at = 4 * (32 * (q / 31) + q % 31);
+      double v[4];
+      for (int e = 0; e < 4; ++e) {
+        v[e] = cl.map_shared_rank(Cs, 0)[at + e];
+        for (int z = 1; z < nz; ++z) v[e] += cl.map_shared_rank(Cs, z)[at + e];
+      }
+      const double* Pq = cl.map_shared_rank(P, q / rows) + 2 * (q % rows);
+      double* o = T + 6 * t;
+      o[0] = Pq[0];
+      o[1] = Pq[1];
+      o[2] = -(v[0] + v[2]);  // A_i = -S_i - B_i
+      o[3] = -(v[1] + v[3]);
+      o[4] = v[2];
+      o[5] = v[3];
+    }
+    cl.sync();  // (a barrier of the block; and no block leaves while others read it)
+    for (int t = tid; t < nr; t += kAdjF64Threads) {
+      const int k = j0 + t, km = (k == 0) ? n - 1 : k - 1;
+      const double *m = T + 6 * t, *o = m + 6;  // panels k - 1 and k
+      double ex, ey, gx, gy;
+      node_terms(nodes, ub, lb, n, k, vinf ? vinf[b] : 1.0, chord ? chord[b] : 1.0, alpha[b], ex,
+                 ey, gx, gy);
+      gx += kInvTwoPi * (0.5 * (lb[km] * m[0] + lb[k] * o[0]) + ub[k] * o[2] + ub[km] * m[4]);
+      gy += kInvTwoPi * (0.5 * (lb[km] * m[1] + lb[k] * o[1]) + ub[k] * o[3] + ub[km] * m[5]);
+      gout[2 * k] = gscale * (ex + gx);
+      gout[2 * k + 1] = gscale * (ey + gy);
+    }
+  } else {
+    for (int k = threadIdx.x; k < nr; k += kAdjF64Threads) {
+      // lambda_j P_j / 2 belongs to the nodes j and j + 1 (the ends of panel j)
+      const int j = j0 + k, j1 = (j + 1 == n) ? 0 : j + 1;
+      const double f = 0.5 * w2pi * lam[k];
+      atomicAdd(&gout[2 * j], f * P[2 * k]);
+      atomicAdd(&gout[2 * j + 1], f * P[2 * k + 1]);
+      atomicAdd(&gout[2 * j1], f * P[2 * k]);
+      atomicAdd(&gout[2 * j1 + 1], f * P[2 * k + 1]);
+    }
   }
 }
 
@@ -432,14 +505,24 @@ cudaError_t launch_adjoint_f64(const Batch& bt, const double* LU, const int32_t*
     if (e != cudaSuccess) return e;
     lam = lambda_out;
   }
+  const int rows = f64_rows(bt.B, bt.n_max), nz = (bt.n_max + rows - 1) / rows;
+  if (bt.n_max <= kFixedF64N) {
+    const size_t smem = ((size_t)rows * 11 + 6 * (rows + 1) + 8 * 32 * 4) * sizeof(double);
+    e = ensure_smem(k_adjoint_f64<true>, smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at;
+    const cudaLaunchConfig_t cfg =
+        cluster_config(dim3(bt.B, nz), dim3(1, nz), kAdjF64Threads, smem, s, &at);
+    return cudaLaunchKernelEx(&cfg, k_adjoint_f64<true>, bt, u, lam, alpha, vinf, chord, grad_cl,
+                              grad, info, rows);
+  }
   e = launch_adjoint_prepare(bt, u, lam, alpha, vinf, chord, grad_cl, grad, info, false, s);
   if (e != cudaSuccess) return e;
-  const int rows = f64_rows(bt.B, bt.n_max);
   const size_t smem = (size_t)rows * 5 * sizeof(double);
-  e = ensure_smem(k_adjoint_f64, smem);
+  e = ensure_smem(k_adjoint_f64<false>, smem);
   if (e != cudaSuccess) return e;
-  k_adjoint_f64<<<dim3(bt.B, (bt.n_max + rows - 1) / rows), kAdjF64Threads, smem, s>>>(
-      bt, u, lam, grad_cl, grad, info, rows);
+  k_adjoint_f64<false><<<dim3(bt.B, nz), kAdjF64Threads, smem, s>>>(
+      bt, u, lam, alpha, vinf, chord, grad_cl, grad, info, rows);
   return cudaGetLastError();
 }
 

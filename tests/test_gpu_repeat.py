@@ -1,5 +1,6 @@
 """Calls that give the same bits in every run: the strengths at every size, and the
-gradients of the sizes whose sums go in a fixed order (up to 256 panels)."""
+gradients of the sizes whose sums go in a fixed order (up to 256 panels in the mixed
+path, up to 64 in the plain FP64 one)."""
 import numpy as np
 import pytest
 
@@ -43,6 +44,19 @@ def test_mixed_gradients_repeat(sizes, batch):
     _same_every_time(step)
     w = torch.as_tensor(np.random.default_rng(1).normal(size=pb.total_nodes))
     _same_every_time(lambda: [pb.vjp(w_cp=w)])
+
+
+@pytest.mark.parametrize("sizes,batch", [((64,), 1), ((40,), 64), ((3, 31, 32, 63, 64), 35),
+                                         ((62,), 400), ((64, 12), 700)])
+def test_fp64_gradients_repeat(sizes, batch):
+    need_gpu()
+    pop, pb = _batch(sizes, batch, mode="fp64")
+
+    def step():
+        pb.run(with_grad=True)
+        return pb.u, pb.lam, pb.grad
+
+    _same_every_time(step)
 
 
 @pytest.mark.parametrize("sizes,batch", [((300, 290), 6), ((700, 400), 20), ((1100,), 3)])
