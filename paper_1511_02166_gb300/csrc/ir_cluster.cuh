@@ -120,7 +120,8 @@ __device__ __forceinline__ float col_part(const CrFactor& f, int d, int t0, int 
 }
 
 struct IrClSmem {
-  double* red;   // 32
+  double* red;   // converged_words
+  double* dprev; // 2
   double* x[2];  // m each
   float *y, *z;  // m: the corrections
   float *xh[2], *xl[2], *r[2];  // m each
@@ -133,7 +134,7 @@ struct IrClSmem {
 
 __host__ __device__ inline size_t ir_cluster_smem(int n_max) {
   const size_t mv = (size_t)n_max + 1;
-  return 32 * 8 + 2 * mv * 8 + 13 * mv * 4 + 2 * 8 * 32 * 4 + 2 * 4 * 32 * 4 + 16 +
+  return (size_t)(converged_words(kIrClThreads) + 2) * 8 + 2 * mv * 8 + 13 * mv * 4 + 2 * 8 * 32 * 4 + 2 * 4 * 32 * 4 + 16 +
          (size_t)kIrClSlots * 32 * sizeof(ResAcc);
 }
 
@@ -354,7 +355,8 @@ __global__ void __launch_bounds__(kIrClThreads, 1) k_ir_cluster(SolveArgs a) {
   const int mv = bt.n_max + 1;
   IrClSmem sm;
   sm.red = reinterpret_cast<double*>(smraw);
-  sm.x[0] = sm.red + 32;
+  sm.dprev = sm.red + converged_words(kIrClThreads);
+  sm.x[0] = sm.dprev + 2;
   sm.x[1] = sm.x[0] + mv;
   float* fp = reinterpret_cast<float*>(sm.x[1] + mv);
   sm.y = fp;
@@ -394,8 +396,6 @@ __global__ void __launch_bounds__(kIrClThreads, 1) k_ir_cluster(SolveArgs a) {
   cl.sync();  // every block of the cluster runs before its memory is written
 
   bool conv[2] = {!act[0], !act[1]};
-  float dprev[2] = {0.0f, 0.0f};
-  const float tol = (float)a.tol;
   int it = 0;
   for (;; ++it) {
     const bool run[2] = {!conv[0], !conv[1]};
@@ -410,11 +410,12 @@ __global__ void __launch_bounds__(kIrClThreads, 1) k_ir_cluster(SolveArgs a) {
       cluster_sweeps(cl, crf, run[0], run[1], sm, m, C, rank);
     else
       cluster_sweeps(cl, RmFactor{F, m}, run[0], run[1], sm, m, C, rank);
+    unsigned long long dm[2] = {0, 0}, xm[2] = {0, 0};
+#pragma unroll
     for (int q = 0; q < 2; ++q) {
       if (!run[q]) continue;
       const float* w = (q == 0) ? sm.y : sm.z;
       double* x = sm.x[q];
-      float dmax = 0.0f, xmax = 0.0f;
       for (int k = tid; k < m; k += kIrClThreads) {
         const int dst = (q == 0) ? k : sm.perm[k];
         const double d = (dst == n) ? (double)w[k] * s : (double)w[k];
@@ -423,16 +424,11 @@ __global__ void __launch_bounds__(kIrClThreads, 1) k_ir_cluster(SolveArgs a) {
         const df2 v = df_from_double(xn);
         sm.xh[q][dst] = v.hi;
         sm.xl[q][dst] = v.lo;
-        dmax = fmaxf(dmax, fabsf((float)d));
-        xmax = fmaxf(xmax, fabsf(v.hi));
+        dm[q] = max(dm[q], magnitude_bits(d));
+        xm[q] = max(xm[q], magnitude_bits(xn));
       }
-      block_max2(dmax, xmax, sm.red);
-      // the stopping rule of k_ir_mixed
-      if (it >= 2 && dmax <= tol * xmax) conv[q] = true;
-      if (it >= 2 && dmax <= 0.125f * dprev[q] && dmax * (dmax / dprev[q]) <= tol * xmax)
-        conv[q] = true;
-      dprev[q] = dmax;
     }
+    block_converged(dm, xm, run, it, a.tol, sm.dprev, conv, sm.red);  // as in k_ir_mixed
     if ((conv[0] && conv[1]) || it >= a.max_iter) break;
     if (it == 0)
       cluster_residuals<LiteAcc>(cl, Ah, Al, m, !conv[0], !conv[1], rhs[0], rhs[1], sm, C, rank);

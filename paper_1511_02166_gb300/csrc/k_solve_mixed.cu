@@ -1640,9 +1640,9 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
   if (a.info[b] != 0 || n > bt.n_max) return;
   const int mv = bt.n_max + 1;
   using RT = typename std::conditional<KEEP, double, float>::type;
-  double* red = reinterpret_cast<double*>(smraw);  // 32
+  double* red = reinterpret_cast<double*>(smraw);
   IrSystem<RT> sys[2];
-  double* dp = red + 32;
+  double* dp = red + converged_words(NT);
   double* bbs = dp;  // KEEP: x, r, bb of both systems (6 m doubles)
   if (KEEP) {
     for (int q = 0; q < 2; ++q) {
@@ -1668,8 +1668,9 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
   float* t32 = reinterpret_cast<float*>(perm + mv);  // 32
   // per-warp partial sums: of the inverse's products (floats, m <= kGjM), or of
   // the fused residual pass (ResAcc, launches with n_max + 1 <= kFuseM)
+  double* dprev = reinterpret_cast<double*>(t32 + 32);  // 2
   float* part = reinterpret_cast<float*>(
-      (reinterpret_cast<uintptr_t>(t32 + 32) + 15) & ~(uintptr_t)15);
+      (reinterpret_cast<uintptr_t>(dprev + 2) + 15) & ~(uintptr_t)15);
   // The corrections: the forward one in y, the transposed one in z, which is
   // the transposed system's float copy of lambda (rewritten from lambda before
   // it is read again); the transposed sweeps' 64-float group scratch is `red`
@@ -1723,8 +1724,6 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
 
   bool active[2] = {act0, act1};
   bool conv[2] = {!act0, !act1};
-  float dprev[2] = {0.0f, 0.0f};  // size of the previous correction
-  const float tol = (float)a.tol;
   int it = 0;
   for (;; ++it) {
     const bool run0 = active[0] && !conv[0], run1 = active[1] && !conv[1];
@@ -1749,31 +1748,23 @@ __global__ void __launch_bounds__(NT, MINB) k_ir_mixed(SolveArgs a) {
     } else {
       lu_solve<false, 1024 / NT>(RmFactor{F, m}, run0, run1, y, z, t32, t32z);
     }
+    unsigned long long dm[2] = {0, 0}, xm[2] = {0, 0};
+#pragma unroll
     for (int q = 0; q < 2; ++q) {
       if (!(q == 0 ? run0 : run1)) continue;
       IrSystem<RT>& S = sys[q];
       const float* w = (q == 0) ? y : z;
-      float dmax = 0.0f, xmax = 0.0f;
       for (int k = threadIdx.x; k < m; k += (int)blockDim.x) {
         const int dst = (q == 0) ? k : perm[k];
         const double d = (dst == n) ? (double)w[k] * s : (double)w[k];
         const double xn = S.x[dst] + d;
         S.x[dst] = xn;
-        dmax = fmaxf(dmax, fabsf((float)d));
-        xmax = fmaxf(xmax, fabsf((float)xn));
+        dm[q] = max(dm[q], magnitude_bits(d));
+        xm[q] = max(xm[q], magnitude_bits(xn));
       }
-      block_max2(dmax, xmax, red);
-      // Converged when the correction just applied is below tol |x|, or when
-      // the contraction seen over the last two corrections (rho = |d_k| /
-      // |d_{k-1}| <= 1/8) predicts the next one, |d_k| rho, below tol |x|: the
-      // error left in x_{k+1} is about that next correction.
-      // (the correction of iteration 1 comes from the double-float residual,
-      // so the first test waits for iteration 2)
-      if (it >= 2 && dmax <= tol * xmax) conv[q] = true;
-      if (it >= 2 && dmax <= 0.125f * dprev[q] && dmax * (dmax / dprev[q]) <= tol * xmax)
-        conv[q] = true;
-      dprev[q] = dmax;
     }
+    const bool run[2] = {run0, run1};
+    block_converged(dm, xm, run, it, a.tol, dprev, conv, red);
     if ((conv[0] && conv[1]) || it >= a.max_iter) break;
     for (int q = 0; q < 2; ++q) {
       if (!active[q] || conv[q]) continue;
@@ -1834,7 +1825,7 @@ size_t ir_mixed_smem(int n_max, int nt) {
                                              : (size_t)(nt / 32) * kGjM * sizeof(float);
   // x, r and the right-hand side of both systems as doubles (KEEP), or r as floats
   const size_t vecs = (mv <= (size_t)kFuseM) ? 6 * mv * 8 + 5 * mv * 4 : 7 * mv * 4;
-  return 32 * 8 + vecs + mv * 4 + 32 * 4 + 32 + part;
+  return (size_t)converged_words(nt) * 8 + vecs + mv * 4 + 32 * 4 + 32 + part;
 }
 
 }  // namespace panel

@@ -44,23 +44,81 @@ struct SolveArgs {
   const double* u_in;  // [sum m_b]
 };
 
-// Block-wide maxima of two non-negative floats, in place (`red`: 64 words of shared
-// memory; all threads call it).  The sizes a stopping rule compares need no FP64: in
-// doubles, with every thread taking the maximum over the warps, they were 12 % of a
-// 100-panel refinement.
-__device__ __forceinline__ void block_max2(float& a, float& b, double* red) {
+// Magnitude of an FP64 value as an integer that orders like it (0 for NaN, which a
+// maximum passes over).
+__device__ __forceinline__ unsigned long long magnitude_bits(double v) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
+  return u <= 0x7ff0000000000000ull ? u : 0ull;
+}
+__device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(v >> 32) == hi ? (unsigned)v : 0u);
+  return ((unsigned long long)hi << 32) | lo;
+}
+
+// The refinement's stopping test of the systems q with run[q], by the whole block:
+// dm[q], xm[q] are the thread's maxima (magnitude_bits) of the correction just applied
+// and of the solution; dprev is the test's own memory (2 shared words); conv[q] is set once
+// system q has converged.  red: 4 words of 64 bits per warp and one more.
+// Converged when the correction just applied is below tol |x|, or when the contraction
+// seen over the last two corrections (rho = |d_k| / |d_{k-1}| <= 1/8) predicts the next
+// one, |d_k| rho, below tol |x|: the error left in x_{k+1} is about that next
+// correction.  The correction of iteration 1 comes from the double-float residual, so
+// the first test waits for iteration 2, and the sizes before iteration 1 are not needed.
+// Ends with a barrier of the block.
+// Sizes, tolerance and rule are FP64; only the maxima go over the integer pipe, and the
+// rule is one warp's work per system, without the division: FP64 maxima in every thread
+// were 12 % of a 100-panel refinement.  (Corrections pass through float32, so their
+// squares neither overflow nor underflow in FP64.)
+__device__ __forceinline__ void block_converged(const unsigned long long (&dm)[2],
+                                                const unsigned long long (&xm)[2],
+                                                const bool (&run)[2], int it, double tol,
+                                                double* dprev, bool (&conv)[2], double* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  unsigned* w = reinterpret_cast<unsigned*>(red);
-  const unsigned ua = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
-  const unsigned ub = __reduce_max_sync(0xffffffffu, __float_as_uint(b));
-  __syncthreads();
-  if (lane == 0) {
-    w[warp] = ua;
-    w[32 + warp] = ub;
+  if (it == 0) {
+    __syncthreads();
+    return;
   }
+  unsigned long long* w = reinterpret_cast<unsigned long long*>(red);
+  int* flag = reinterpret_cast<int*>(w + 4 * nw);
+  unsigned long long d[2] = {0, 0}, x[2] = {0, 0};
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    if (run[q]) {
+      d[q] = warp_max_u64(dm[q]);
+      x[q] = warp_max_u64(xm[q]);
+    }
+  __syncthreads();  // (red may still be in use)
+  if (lane == 0)
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      w[q * nw + warp] = d[q];
+      w[(2 + q) * nw + warp] = x[q];
+    }
   __syncthreads();
-  a = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < nw ? w[lane] : 0u));
-  b = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < nw ? w[32 + lane] : 0u));
+  if (warp < 2 && (warp == 0 ? run[0] : run[1])) {
+    const double dmax = __longlong_as_double(
+        (long long)warp_max_u64(lane < nw ? w[warp * nw + lane] : 0ull));
+    if (it >= 2) {
+      const double lim = tol * __longlong_as_double((long long)warp_max_u64(
+                                   lane < nw ? w[(2 + warp) * nw + lane] : 0ull));
+      const double dp = dprev[warp];
+      const bool c = dmax <= lim || (dmax <= 0.125 * dp && dmax * dmax <= lim * dp);
+      if (lane == 0) flag[warp] = c ? 1 : 0;
+    }
+    __syncwarp();
+    if (lane == 0) dprev[warp] = dmax;
+  }
+  if (it == 1) return;
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < 2; ++q)
+    if (run[q] && flag[q] != 0) conv[q] = true;
+}
+// Doubles of block_converged's scratch in a block of nt threads (block_sum needs 32; a
+// whole number of 16-byte words).
+__host__ __device__ constexpr int converged_words(int nt) {
+  return nt / 8 + 2 > 32 ? nt / 8 + 2 : 32;
 }
 
 // border scale s = mean |A_jj| over the influence block (hi plane)
