@@ -45,62 +45,80 @@ namespace panel {
 // warp, register-resident: lane r holds row r (x = its 32 columns, zero beyond
 // the block); rows keep their lanes and `pos` tracks their current position, so
 // an exchange of positions q and p is bookkeeping plus one ipiv entry.  The
-// pivot of column q is the largest |x_q| (to 2^-18 of it) among the rows not yet
-// pivotal, the lowest row among equals.
+// pivot of column q is the largest |x_q| among the rows not yet pivotal, the
+// lowest lane (row of the block before its exchanges) among equals.
 //
 // One warp walks a chain of kb dependent steps, so a step's latency is what
-// counts.  One REDUX finds value and lane of the pivot together (the lane in the
-// low five bits of the key); every lane takes the reciprocal of its own entry
-// while the reduction runs, and the pivot's comes by a shuffle.  The columns
-// rotate down the registers as they are updated (x[0] is the current one), so
-// that the step loop stays rolled with constant register indices; each finished
-// entry goes to the row's own place in `blk`.  Four groups of eight steps
-// narrow the update from 31 to 7 columns.  193 cycles a step (one warp alone);
-// 390 with a vote for the lane, the rounded reciprocal (__frcp_rn, ~190 cycles)
-// and entries kept in registers by selects; 285 with the pivot row broadcast
-// through shared memory; 180 without any pivot search.
+// counts.  The next column is brought up to date first, and its pivot searched (a
+// REDUX for the magnitude, a vote for the lane; every lane takes the reciprocal of its
+// own entry) between the updates of the other columns: one airfoil of 200 panels, in
+// shared memory, 88 us (91 with a search of 18-bit magnitudes, the lane in the key's
+// low bits, at the head of the step), of 100, through L2, 39 (40).  A REDUX more, for
+// the lowest position among equals, took 96 and 43 us, a branch for it 92 and 43.
+// The columns rotate down the registers as they are updated (x[0] is the current
+// one), so that the step loop stays rolled with constant register indices; each
+// finished entry goes to the row's own place in `blk`.  Four groups of eight steps
+// narrow the update from 31 to 7 columns.
 // ipiv[q] receives base + the position of column q's pivot row.  On return `fz`
 // is 0, or q + 1 for the first exactly zero (or NaN) pivot column q, after which
 // the block's contents have no meaning.
 // ---------------------------------------------------------------------------
-// 1 / a by one Newton-Raphson step on the hardware approximation.
+// 1 / a by one Newton-Raphson step on the hardware approximation: the correctly
+// rounded reciprocal for every |a| below 2^126, infinite ones included (compared with
+// __frcp_rn on all of them; beyond, where it is subnormal, 5 magnitudes differ in the
+// last bit).
 __device__ __forceinline__ float rcp_newton(float a) {
   float r;
   asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return fmaf(r, fmaf(-a, r, 1.0f), r);
+  const float v = fmaf(r, fmaf(-a, r, 1.0f), r);
+  return v == v ? v : r;
 }
+
+// The pivot of a column, x the lane's entry: largest() and vote(), apart (a warp keeps
+// the order of such operations, and the second waits for the first).
+struct PivotSearch {
+  unsigned key, mx;  // the lane's magnitude (0: no candidate), the largest
+  int lane;
+  float rcp;         // of the lane's own entry
+  __device__ __forceinline__ void largest(float x, bool done) {
+    key = (!done && x == x) ? __float_as_uint(x) & 0x7fffffffu : 0u;
+    mx = __reduce_max_sync(0xffffffffu, key);
+    rcp = rcp_newton(x);
+  }
+  __device__ __forceinline__ void vote() {
+    lane = __ffs(__ballot_sync(0xffffffffu, key == mx)) - 1;
+  }
+};
 
 template <int W, class Blk>
 __device__ __forceinline__ void warp_block_lu_group(float (&x)[32], const Blk& blk, int& pos,
                                                     bool& done, int& fz, int kb, int* ipiv,
-                                                    int base) {
+                                                    int base, PivotSearch& s) {
   const int lane = threadIdx.x & 31;
 #pragma unroll 1
   for (int lq = 0; lq < 8; ++lq) {
     const int q = 32 - W + lq;
-    const unsigned bits = __float_as_uint(x[0]) & 0x7fffffe0u;  // |x|, monotone
-    const unsigned key = (!done && x[0] == x[0]) ? bits | (31u - lane) : 0u;
-    const float rcp = rcp_newton(x[0]);
-    const unsigned mx = __reduce_max_sync(0xffffffffu, key);
-    const int pl = 31 - (int)(mx & 31u);
-    const bool ok = mx > 31u;  // a nonzero pivot
-    const float inv = __shfl_sync(0xffffffffu, rcp, pl);
-    const float l = x[0] * inv;
+    const int pl = s.lane;
+    const bool ok = s.mx != 0u;  // a nonzero pivot
+    const float l = x[0] * __shfl_sync(0xffffffffu, s.rcp, pl);
     const bool elim = ok && !done && lane != pl;
     const float le = elim ? l : 0.0f;
     if (lane < kb && q < kb) blk(lane, q) = elim ? l : x[0];
+    if (ok && lane == pl) done = true;
+    x[0] = fmaf(-le, __shfl_sync(0xffffffffu, x[1], pl), x[1]);
+    s.largest(x[0], done);
 #pragma unroll
-    for (int t = 1; t < W; ++t) x[t - 1] = fmaf(-le, __shfl_sync(0xffffffffu, x[t], pl), x[t]);
+    for (int t = 2; t < W; ++t) {
+      x[t - 1] = fmaf(-le, __shfl_sync(0xffffffffu, x[t], pl), x[t]);
+      if (t == (W < 16 ? W - 2 : 14)) s.vote();
+    }
     x[W - 1] = 0.0f;
     // bookkeeping, off the chain
     const int pm = __shfl_sync(0xffffffffu, pos, pl);
     if (ok) {
       if (lane == 0) ipiv[q] = base + pm;
       if (pos == q) pos = pm;
-      if (lane == pl) {
-        pos = q;
-        done = true;
-      }
+      if (lane == pl) pos = q;
     } else if (q < kb && fz == 0) {
       fz = q + 1;
     }
@@ -110,10 +128,13 @@ __device__ __forceinline__ void warp_block_lu_group(float (&x)[32], const Blk& b
 template <class Blk>
 __device__ __forceinline__ void warp_block_lu(float (&x)[32], const Blk& blk, int& pos, bool& done,
                                               int& fz, int kb, int* ipiv, int base) {
-  warp_block_lu_group<32>(x, blk, pos, done, fz, kb, ipiv, base);
-  if (kb > 8) warp_block_lu_group<24>(x, blk, pos, done, fz, kb, ipiv, base);
-  if (kb > 16) warp_block_lu_group<16>(x, blk, pos, done, fz, kb, ipiv, base);
-  if (kb > 24) warp_block_lu_group<8>(x, blk, pos, done, fz, kb, ipiv, base);
+  PivotSearch s;
+  s.largest(x[0], done);
+  s.vote();
+  warp_block_lu_group<32>(x, blk, pos, done, fz, kb, ipiv, base, s);
+  if (kb > 8) warp_block_lu_group<24>(x, blk, pos, done, fz, kb, ipiv, base, s);
+  if (kb > 16) warp_block_lu_group<16>(x, blk, pos, done, fz, kb, ipiv, base, s);
+  if (kb > 24) warp_block_lu_group<8>(x, blk, pos, done, fz, kb, ipiv, base, s);
 }
 
 // ---------------------------------------------------------------------------
