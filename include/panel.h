@@ -281,6 +281,18 @@ int panel_adjoint(int B, int n_max, int flags, const double* nodes, const int64_
                   int32_t* info, void* stream);
 
 /*
+ * panel_launches -- kernels that one call launches for B airfoils of at most n_max
+ *   panels with these flags (tuning fields included) on a device of sms
+ *   multiprocessors: PANEL_CALL_ASSEMBLE, PANEL_CALL_SOLVE, or PANEL_CALL_ADJOINT
+ *   with a given lambda.  By the rules the launches themselves go by; host only.
+ *   -PANEL_EINVAL for arguments that the calls refuse, or sms < 1.
+ */
+#define PANEL_CALL_ASSEMBLE 0
+#define PANEL_CALL_SOLVE 1
+#define PANEL_CALL_ADJOINT 2
+int panel_launches(int call, int B, int n_max, int flags, int sms);
+
+/*
  * panel_polar -- Cl at K angles of attack per airfoil from one factorisation
  * (PANEL_MIXED only; PANEL_FP64 returns PANEL_ENOTSUP).
  *   The right-hand side of Section 2's system is linear in (cos a, sin a):

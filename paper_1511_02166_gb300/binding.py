@@ -75,6 +75,7 @@ SIGNATURES = {
                            _P]),
     "panel_adjoint": (_I, [_I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
                            _P, _P, _P, _I, _D, _P, _P]),
+    "panel_launches": (_I, [_I, _I, _I, _I, _I]),
     "panel_polar": (_I, [_I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _I, _P, _P, _P,
                          _P, _I, _D, _P, _P, _P]),
     "panel_vjp": (_I, [_I, _I, _I, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P, _P,
@@ -208,6 +209,17 @@ def panel_adjoint(B, n_max, flags, nodes, node_offsets, mat_offsets, order, A64,
                                 _ptr(lambda_out), _ptr(alpha), _ptr(vinf), _ptr(chord),
                                 _ptr(grad_cl), _ptr(grad_nodes), int(max_iter), float(tol),
                                 _ptr(info), _stream(stream)), "panel_adjoint")
+
+
+CALL_ASSEMBLE, CALL_SOLVE, CALL_ADJOINT = 0, 1, 2
+
+
+def panel_launches(call, B, n_max, flags, sms) -> int:
+    """Host: kernels of one call (CALL_*) of B airfoils of at most n_max panels with
+    these flags on a device of `sms` multiprocessors."""
+    n = load().panel_launches(int(call), int(B), int(n_max), int(flags), int(sms))
+    _check(max(-n, 0), "panel_launches")
+    return n
 
 
 def panel_viscous(B, nodes, node_offsets, u, alpha, vinf, chord, reynolds, info, cl, ld, cd,

@@ -53,6 +53,10 @@ cudaError_t launch_ir_vjp(const Batch&, const float*, const float*, const float*
                           const int32_t*, const double*, const double*, const double*,
                           const double*, const double*, const double*, double*, int, double,
                           int32_t*, cudaStream_t);
+int assemble_df_launches(int B, int n_max, int sel, int sms);
+int lu_mixed_launches(int B, int n_max, bool inverse, int lu_kind, int sms);
+int adjoint_df_launches(int n_max);
+int adjoint_f64_launches(int n_max);
 }  // namespace panel
 
 using panel::Batch;
@@ -206,6 +210,29 @@ int panel_solve(int B, int n_max, int flags, const double* nodes, const int64_t*
                                adj ? lambda : nullptr, max_iter, tol, info, iters, s, 0,
                                tune_ir(flags));
   return status_of(e);
+}
+
+int panel_launches(int call, int B, int n_max, int flags, int sms) {
+  if (B < 0 || n_max < 3 || n_max > PANEL_N_MAX || !flags_ok(flags) || sms < 1)
+    return -PANEL_EINVAL;
+  const bool f64 = mode_of(flags) == PANEL_FP64;
+  if (B == 0) return 0;
+  switch (call) {
+    case PANEL_CALL_ASSEMBLE:
+      return f64 ? 1 : panel::assemble_df_launches(B, n_max, tune_rounds(flags), sms);
+    case PANEL_CALL_SOLVE: {
+      if (f64) return 1;
+      const int factor = (flags & PANEL_REUSE_FACTOR)
+                             ? 0
+                             : panel::lu_mixed_launches(B, n_max, (flags & PANEL_INVERSE) != 0,
+                                                        tune_lu(flags), sms);
+      return factor + ((flags & PANEL_FACTOR_ONLY) ? 0 : 1);
+    }
+    case PANEL_CALL_ADJOINT:
+      return f64 ? panel::adjoint_f64_launches(n_max) : panel::adjoint_df_launches(n_max);
+    default:
+      return -PANEL_EINVAL;
+  }
 }
 
 int panel_polar(int B, int n_max, int flags, const double* nodes, const int64_t* node_offsets,

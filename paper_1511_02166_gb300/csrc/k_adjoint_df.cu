@@ -796,6 +796,9 @@ cudaError_t launch_adjoint_prepare(const Batch& bt, const double* u, const doubl
   return cudaGetLastError();
 }
 
+// Kernels of launch_adjoint_df.
+int adjoint_df_launches(int n_max) { return n_max > kPartialsN ? 2 : 1; }
+
 cudaError_t launch_adjoint_df(const Batch& bt, const double* u, const double* lambda,
                               const double* alpha, const double* vinf, const double* chord,
                               const double* grad_cl, double* grad, const int32_t* info,

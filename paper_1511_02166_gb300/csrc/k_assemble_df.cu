@@ -437,11 +437,11 @@ static size_t assemble_df_smem(int n_max, int rounds) {
 // one block per airfoil is best for many airfoils of few panels, where most warps
 // hold near-field pairs; the pair-at-once tiles everywhere else.
 enum AssembleKind { kAsmBlock, kAsmSplit, kAsmTiles64, kAsmTiles128 };
-static AssembleKind assemble_kind(int B, int n_max, int sel) {
+static AssembleKind assemble_kind(int B, int n_max, int sel, int sm_total) {
   if (sel >= 1 && sel <= 5) return kAsmBlock;
   if (sel == 6) return kAsmTiles128;
   if (n_max <= 64) return kAsmBlock;
-  const long long sms = sm_count() > 0 ? sm_count() : 1;
+  const long long sms = sm_total > 0 ? sm_total : 1;
   auto pairs = [&](int c) {
     const long long nch = (n_max + c - 1) / c;
     return B * (nch * (nch + 1) / 2);
@@ -451,10 +451,15 @@ static AssembleKind assemble_kind(int B, int n_max, int sel) {
   return pairs(128) < 3 * sms ? kAsmTiles64 : kAsmTiles128;
 }
 
+// Kernels of launch_assemble_df.
+int assemble_df_launches(int B, int n_max, int sel, int sms) {
+  return assemble_kind(B, n_max, sel, sms) == kAsmBlock ? 1 : 2;
+}
+
 cudaError_t launch_assemble_df(const Batch& bt, const double* alpha, const double* vinf,
                                float* A_hi, float* A_lo, double* rhs, int32_t* info,
                                cudaStream_t s, int rounds_sel) {
-  const AssembleKind kind = assemble_kind(bt.B, bt.n_max, rounds_sel);
+  const AssembleKind kind = assemble_kind(bt.B, bt.n_max, rounds_sel, sm_count());
   if (kind == kAsmBlock) {
     int rounds = assemble_rounds(bt.n_max, rounds_sel);
     // a requested queue that does not fit the shared memory falls back to the default

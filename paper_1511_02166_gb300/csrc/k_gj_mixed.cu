@@ -247,6 +247,8 @@ size_t gj_smem_bytes(int n_max) {
   return mf * (mf | 1) * 4;
 }
 
+int gj_launches(int mv) { return mv > kSmemM ? 2 : 1; }
+
 cudaError_t launch_gj_mixed(const SolveArgs& a, cudaStream_t s) {
   const Batch& bt = a.bt;
   if (!a.inverse) return cudaSuccess;  // the LU takes every airfoil
@@ -256,7 +258,7 @@ cudaError_t launch_gj_mixed(const SolveArgs& a, cudaStream_t s) {
   k_gj_mixed<true><<<bt.B, kThreads, smem, s>>>(a);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (bt.n_max + 1 > kSmemM) {
+  if (gj_launches(bt.n_max + 1) > 1) {
     k_gj_mixed<false><<<bt.B, kThreads, 0, s>>>(a);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -775,6 +775,14 @@ static int split_for(int B, int per_airfoil_max, int per_sm = 4) {
   return max(1, min(want, per_airfoil_max));
 }
 
+// The copy in, T diagonal blocks with T - 1 triangular solves and updates between them,
+// the untransposed U tiles and the finishing pass.
+int lu_large_launches(int mv) {
+  if (mv <= kLargeM) return 0;
+  const int T = (mv + kTlB - 1) / kTlB;
+  return 1 + T + 2 * (T - 1) + ((T - 1) * (T - 2) / 2 > 0 ? 1 : 0) + 1;
+}
+
 cudaError_t launch_lu_large(const SolveArgs& a, cudaStream_t s) {
   const Batch& bt = a.bt;
   const int B = bt.B, m_max = bt.n_max + 1;

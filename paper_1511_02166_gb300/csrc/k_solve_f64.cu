@@ -491,6 +491,9 @@ __global__ void __launch_bounds__(kAdjF64Threads) k_adjoint_f64(
   }
 }
 
+// Kernels of launch_adjoint_f64 with a given lambda.
+int adjoint_f64_launches(int n_max) { return n_max > kFixedF64N ? 2 : 1; }
+
 cudaError_t launch_adjoint_f64(const Batch& bt, const double* LU, const int32_t* piv,
                                const double* u, const double* lambda_in, double* lambda_out,
                                const double* alpha, const double* vinf, const double* chord,

@@ -1891,9 +1891,21 @@ static SolveArgs make_args(const Batch& bt, const float* A_hi, const float* A_lo
 // 160 unknowns, by its shorter steps (1 of 165 panels 69 / 72, of 205 91 / 98; 304 of
 // 165 141 / 93).  A launch that also holds larger airfoils runs them all through L2
 // at once.
-static int lu_kind_by_size(int B, int mv) {
+static int lu_kind_by_size(int B, int mv, int sms) {
   if (mv > kSmemLuM) return 1;
-  return mv <= 64 || (mv > 160 && B <= sm_count()) ? 2 : 1;
+  return mv <= 64 || (mv > 160 && B <= sms) ? 2 : 1;
+}
+// Whether a launch runs k_lu_smem and k_lu_global.
+static bool runs_lu_smem(bool inverse, int lu_kind) { return !inverse && lu_kind != 1; }
+static bool runs_lu_global(int mv, bool inverse, int lu_kind) {
+  return (mv > kSmemLuM || lu_kind == 1) && (mv > kGjM || !inverse);
+}
+// Kernels of launch_lu_mixed.
+int lu_mixed_launches(int B, int n_max, bool inverse, int lu_kind, int sms) {
+  const int mv = n_max + 1;
+  if (lu_kind == 0) lu_kind = lu_kind_by_size(B, mv, sms);
+  return lu_large_launches(mv) + (runs_lu_smem(inverse, lu_kind) ? 1 : 0) +
+         (runs_lu_global(mv, inverse, lu_kind) ? 1 : 0) + (inverse ? gj_launches(mv) : 0);
 }
 
 // Factor every airfoil: with `inverse` the Gauss-Jordan inverse for m <= kGjM;
@@ -1906,14 +1918,14 @@ cudaError_t launch_lu_mixed(const Batch& bt, const float* A_hi, float* LU, int32
   SolveArgs a = make_args(bt, A_hi, nullptr, LU, piv, nullptr, nullptr, nullptr, nullptr,
                           nullptr, 0, 0.0, info, iters);
   a.inverse = inverse ? 1 : 0;
-  if (lu_kind == 0) lu_kind = lu_kind_by_size(bt.B, bt.n_max + 1);
+  if (lu_kind == 0) lu_kind = lu_kind_by_size(bt.B, bt.n_max + 1, sm_count());
   a.lu_kind = lu_kind;
   cudaError_t e;
   if (bt.n_max + 1 > kLargeM) {
     e = launch_lu_large(a, s);
     if (e != cudaSuccess) return e;
   }
-  if (!inverse && lu_kind != 1) {
+  if (runs_lu_smem(inverse, lu_kind)) {
     // airfoils up to kSmemLuM unknowns with the whole matrix in shared memory
     SolveArgs h = a;
     h.bt.n_max = min(bt.n_max, kSmemLuM - 1);
@@ -1929,7 +1941,7 @@ cudaError_t launch_lu_mixed(const Batch& bt, const float* A_hi, float* LU, int32
                  : mv <= 128 ? go(k_lu_smem<256, 3>, 256) : go(k_lu_smem<512, 1>, 512);
     if (e != cudaSuccess) return e;
   }
-  if ((bt.n_max + 1 > kSmemLuM || lu_kind == 1) && (bt.n_max + 1 > kGjM || !inverse)) {
+  if (runs_lu_global(bt.n_max + 1, inverse, lu_kind)) {
     SolveArgs g = a;
     g.bt.n_max = min(bt.n_max, kLargeM - 1);
     const size_t smem = lu_global_smem(g.bt.n_max);

@@ -228,6 +228,9 @@ __device__ __forceinline__ void tri_subst(float (&x)[32], const float* tab, cons
 
 cudaError_t launch_lu_large(const SolveArgs& a, cudaStream_t s);
 cudaError_t launch_gj_mixed(const SolveArgs& a, cudaStream_t s);
+// Kernels of the two for airfoils of at most mv unknowns.
+int lu_large_launches(int mv);
+int gj_launches(int mv);
 long long set_wait_limit(long long polls);
 size_t lu_large_min_m();
 

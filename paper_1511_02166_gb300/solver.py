@@ -84,24 +84,6 @@ GJ_MAX_M = 288  # largest m = n + 1 that the library factors by Gauss-Jordan
 LU_SMEM_MAX_M = 222  # largest m whose LU the library can run in shared memory
 
 
-def assembly_spread(count, n_max, rounds, sms):
-    """Whether the library assembles `count` airfoils of at most n_max panels with
-    several blocks per airfoil (a preparing launch, then the pairs)."""
-    if rounds or n_max <= 64:
-        return rounds == 6
-    nch = -(-n_max // 64)
-    return count * nch * (nch + 1) // 2 <= sms or not (
-        n_max <= 128 or (n_max <= 224 and count > sms))
-
-
-def lu_kind_by_size(count, m, sms):
-    """The one-block LU that the library takes by default for `count` airfoils of
-    at most m unknowns on `sms` multiprocessors (1 through L2, 2 in shared memory)."""
-    if m > LU_SMEM_MAX_M:
-        return 1
-    return 2 if m <= 64 or (m > 160 and count <= sms) else 1
-
-
 def _require_cuda(device):
     dev = torch.device(device)
     if dev.type != "cuda" or not torch.cuda.is_available():
@@ -220,7 +202,7 @@ class PanelBatch:
     def _asm_tune(self, k):
         return bd.PANEL_TUNE_ROUNDS(self.rounds[k]) if self.flags == bd.PANEL_MIXED else 0
 
-    def _solve_bucket(self, k, start, cnt, nmax, with_adjoint, stage, stream=None):
+    def _solve_flags(self, k, with_adjoint, stage):
         f = self.flags | (bd.PANEL_WITH_ADJOINT if with_adjoint else 0)
         f |= {"all": 0, "factor": bd.PANEL_FACTOR_ONLY, "refine": bd.PANEL_REUSE_FACTOR}[stage]
         if self.flags == bd.PANEL_MIXED:
@@ -229,6 +211,10 @@ class PanelBatch:
                 f |= bd.PANEL_TUNE_LU(self.lu_kind[k])
         if self.inverse[k] and stage != "refine":
             f |= bd.PANEL_INVERSE
+        return f
+
+    def _solve_bucket(self, k, start, cnt, nmax, with_adjoint, stage, stream=None):
+        f = self._solve_flags(k, with_adjoint, stage)
         bd.panel_solve(cnt, nmax, f, self.nodes, self.node_offsets, self.mat_offsets,
                        self.order[start:], self.A64, self.A_hi, self.A_lo, self.LU,
                        self.piv, self.rhs, self.vinf, self.chord, self.u,
@@ -338,37 +324,16 @@ class PanelBatch:
             self.run(with_grad=with_grad)
 
     def launches_per_step(self, with_grad: bool = True) -> int:
-        """Kernel launches of one step: per bucket assemble (two when the pairs are
-        spread over several blocks per airfoil), factor, refine and adjoint, plus
-        one forces launch.  The mixed factor launches one kernel
-        per size class the bucket may hold (Gauss-Jordan in shared memory and in
-        global memory, or the one-block LU in shared memory and through L2) and,
-        for m > 640 with T 128-column blocks, the step-synchronous LU: the tiled
-        copy, T diagonal LUs, one CUDA-core and T - 1 tensor-core triangular
-        solves, T - 1 updates, the untranspose of the U tiles and the inversion
-        of the diagonal blocks; the split adjoint (n > 256, or fewer 32-column warps
-        than eight per SM) adds a launch for the terms without pair sums."""
-        n = 1  # forces
+        """Kernel launches of one step: per bucket those of assemble, solve and
+        adjoint (as the library counts them), plus one forces launch."""
         sms = torch.cuda.get_device_properties(self.device).multi_processor_count
+        n = 1  # forces
         for k, (start, cnt, nmax) in enumerate(self.buckets):
-            m = nmax + 1
-            n += 1 + (self.flags == bd.PANEL_MIXED and
-                      assembly_spread(cnt, nmax, self.rounds[k], sms))
-            if self.flags == bd.PANEL_MIXED:
-                if self.inverse[k]:
-                    n += 1 + (m > 230) + (m > GJ_MAX_M)
-                else:
-                    kind = self.lu_kind[k] or lu_kind_by_size(cnt, m, sms)
-                    n += (kind != 1) + (m > LU_SMEM_MAX_M or kind == 1)
-                if m > 640:
-                    blocks = -(-m // 128)
-                    n += 3 + blocks + 2 * (blocks - 1)
-                n += 1  # refine
-            else:
-                n += 1
+            n += bd.panel_launches(bd.CALL_ASSEMBLE, cnt, nmax, self.flags | self._asm_tune(k), sms)
+            n += bd.panel_launches(bd.CALL_SOLVE, cnt, nmax,
+                                   self._solve_flags(k, with_grad, "all"), sms)
             if with_grad:
-                split = nmax > 256 or cnt * (-(-nmax // 32)) < 8 * sms
-                n += 1 + (split and self.flags == bd.PANEL_MIXED)
+                n += bd.panel_launches(bd.CALL_ADJOINT, cnt, nmax, self.flags, sms)
         return n
 
     # -- autotuning and graph capture -------------------------------------------
