@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import concurrent.futures as cf
 import glob
+import hashlib
 import os
 import shutil
 import subprocess
@@ -35,6 +36,15 @@ def _sources():
 def _deps():
     return _sources() + sorted(glob.glob(os.path.join(CSRC, "*.cuh"))) + [
         os.path.join(ROOT, "include", "panel.h"), os.path.abspath(__file__)]
+
+
+def source_key() -> str:
+    """Identifies the sources the library is built from (12 hexadecimal digits)."""
+    h = hashlib.sha1()
+    for path in _deps():
+        with open(path, "rb") as f:
+            h.update(os.path.basename(path).encode() + b"\0" + f.read() + b"\0")
+    return h.hexdigest()[:12]
 
 
 def up_to_date() -> bool:

@@ -22,6 +22,7 @@ import numpy as np
 import torch
 
 from . import binding as bd
+from . import build
 
 _tune_lock = threading.Lock()
 
@@ -82,6 +83,23 @@ def size_buckets(sorted_sizes, width, min_count=1):
 MODES = {"fp64": bd.PANEL_FP64, "mixed": bd.PANEL_MIXED}
 GJ_MAX_M = 288  # largest m = n + 1 that the library factors by Gauss-Jordan
 LU_SMEM_MAX_M = 222  # largest m whose LU the library can run in shared memory
+
+
+def tuning_class(count, sms):
+    """Batches that share an autotuned choice: the dispatch rules depend on the exact
+    count up to eight airfoils per multiprocessor, and not on it above."""
+    return min(int(count), 8 * sms)
+
+
+def solve_candidates(n_max):
+    """(inverse, LU kind) pairs that the autotuner times for airfoils of at most n_max
+    panels, the library's own choice first: a later one has to be 1 % faster."""
+    factors = [(False, 0)]
+    if n_max + 1 <= LU_SMEM_MAX_M:
+        factors += [(False, 2), (False, 1)]
+    if n_max + 1 <= GJ_MAX_M:
+        factors.append((True, 0))
+    return factors
 
 
 def _require_cuda(device):
@@ -358,18 +376,18 @@ class PanelBatch:
           2. per bucket, the assembly (PANEL_TUNE_ROUNDS 0..6: near-field rounds, or
              both entries of a pair at once);
           3. per bucket, the solve (factor + refinement of both systems): the LU
-             (for m <= 222 with the matrix in shared memory or through L2,
-             PANEL_TUNE_LU 2 / 1) or the Gauss-Jordan inverse (m <= 288), each
+             (the library's choice, and for m <= 222 the matrix in shared memory or
+             through L2, PANEL_TUNE_LU 2 / 1) or the Gauss-Jordan inverse (m <= 288), each
              with each refinement block shape (PANEL_TUNE_IR 0..5).
-        Choices are cached by device, size bound and batch class
+        Choices are cached by device, library sources, size bound and batch class
         ($PANEL_AUTOTUNE_CACHE).  Returns {key: choice}."""
         if self.flags != bd.PANEL_MIXED or not self.buckets:
             return dict()
-        dev = torch.cuda.get_device_name(self.device)
+        dev = "%s|%s" % (torch.cuda.get_device_name(self.device), build.source_key())
+        sms = torch.cuda.get_device_properties(self.device).multi_processor_count
         with _tune_lock:
             cache = _load_tune_cache() if use_cache else {}
         chosen = {}
-        bclass = lambda cnt: min(cnt, 1024) // 152 * 152
         sizes = np.diff(self.offsets_h)
         # 1. bucket width
         if len(set(sizes.tolist())) > 1 and widths:
@@ -390,7 +408,7 @@ class PanelBatch:
         torch.cuda.synchronize(self.device)
         for k, (start, cnt, nmax) in enumerate(self.buckets):
             # 2. assembly rounds
-            key = "%s|asm-rounds|n%d|b%d" % (dev, nmax, bclass(cnt))
+            key = "%s|asm-rounds|n%d|b%d" % (dev, nmax, tuning_class(cnt, sms))
             if key not in cache:
                 times = []
                 for r in range(7):
@@ -411,13 +429,10 @@ class PanelBatch:
             self.rounds[k] = int(cache[key])
             chosen[key] = self.rounds[k]
             # 3. factorisation and refinement shape
-            key = "%s|solve-lu|n%d|b%d" % (dev, nmax, bclass(cnt))
+            key = "%s|solve-lu|n%d|b%d" % (dev, nmax, tuning_class(cnt, sms))
             if key not in cache:
                 best, best_t = None, None
-                factors = [(False, 2), (False, 1)] if nmax + 1 <= LU_SMEM_MAX_M else [(False, 0)]
-                if nmax + 1 <= GJ_MAX_M:
-                    factors.append((True, 0))
-                for inverse, lu in factors:
+                for inverse, lu in solve_candidates(nmax):
                     for shape in range(6):
                         f = (bd.PANEL_MIXED | bd.PANEL_WITH_ADJOINT | bd.PANEL_TUNE_IR(shape) |
                              (bd.PANEL_INVERSE if inverse else bd.PANEL_TUNE_LU(lu)))
