@@ -225,9 +225,12 @@ inline int sm_count() {
 // Rows per block of the plain FP64 pair kernels (launched for B airfoils of at most m
 // rows): all of them for a batch of four blocks per SM, else as few as spread the
 // batch over that many blocks, at least 12 (a block's own preparation costs about three
-// rows).
+// rows).  Airfoils of fewer than 24 rows stay whole from three blocks per SM on: 12 rows
+// and a remainder prepare twice for little (456 of 20 panels, assembly 86 us, whole 53).
 inline int f64_rows(int B, int m) {
-  const long long want = 4ll * (sm_count() > 0 ? sm_count() : 1);
+  const int sms = sm_count() > 0 ? sm_count() : 1;
+  if (m < 24 && B > 2 * sms) return m;
+  const long long want = 4ll * sms;
   const long long z = (want + B - 1) / (B > 0 ? B : 1);
   const long long rows = (m + z - 1) / z;
   return (int)(rows < 12 ? (m < 12 ? m : 12) : rows);
