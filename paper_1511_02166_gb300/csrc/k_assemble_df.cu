@@ -435,7 +435,8 @@ static size_t assemble_df_smem(int n_max, int rounds) {
 //   152 x 1024  2729 / 1750 / 1421 / 1369
 // The split kernel fills the chip when even tiles of 64 leave SMs without a block;
 // one block per airfoil is best for many airfoils of few panels, where most warps
-// hold near-field pairs; the pair-at-once tiles everywhere else.
+// hold near-field pairs (one block / tiles of 64: 128 x 140  75 / 76, 140 x 140  74 / 81,
+// 140 x 160  91 / 80); the pair-at-once tiles everywhere else.
 enum AssembleKind { kAsmBlock, kAsmSplit, kAsmTiles64, kAsmTiles128 };
 static AssembleKind assemble_kind(int B, int n_max, int sel, int sm_total) {
   if (sel >= 1 && sel <= 5) return kAsmBlock;
@@ -447,8 +448,9 @@ static AssembleKind assemble_kind(int B, int n_max, int sel, int sm_total) {
     return B * (nch * (nch + 1) / 2);
   };
   if (pairs(64) <= sms) return kAsmSplit;
-  if (n_max <= 128 || (n_max <= 224 && B > sms)) return kAsmBlock;
-  return pairs(128) < 3 * sms ? kAsmTiles64 : kAsmTiles128;
+  if (n_max <= 128 || (n_max <= 144 && 4 * B > 3 * sms) || (n_max <= 224 && B > sms))
+    return kAsmBlock;
+  return pairs(128) <= 3 * sms ? kAsmTiles64 : kAsmTiles128;
 }
 
 // Kernels of launch_assemble_df.

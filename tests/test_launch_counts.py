@@ -19,6 +19,9 @@ COUNTS = [
     (bd.CALL_ASSEMBLE, 51, 128, MIXED, 1),
     (bd.CALL_ASSEMBLE, SMS + 1, 224, MIXED, 1),
     (bd.CALL_ASSEMBLE, SMS + 1, 225, MIXED, 2),
+    (bd.CALL_ASSEMBLE, 114, 144, MIXED, 2),
+    (bd.CALL_ASSEMBLE, 115, 144, MIXED, 1),
+    (bd.CALL_ASSEMBLE, 115, 145, MIXED, 2),
     (bd.CALL_ASSEMBLE, 1, 160, MIXED | bd.PANEL_TUNE_ROUNDS(1), 1),
     (bd.CALL_ASSEMBLE, 4096, 200, MIXED | bd.PANEL_TUNE_ROUNDS(6), 2),
     # factor and refinement
