@@ -1995,17 +1995,16 @@ static int ir_cluster_capacity(int C) {
 
 // Blocks per airfoil of a refinement by clusters, or 0 for k_ir_mixed: the most that
 // let every airfoil of the batch run at once.  Measured, both systems (us, the best
-// block shape of k_ir_mixed / clusters): 1 airfoil of 200 panels 169 / 203; of 256 228 /
-// 257; of 300 324 / 295 (8 blocks); of 600 797 / 577; of 1024 3581 (one block of 1024
-// threads) / 2444, 1589, 1310 (2, 4, 8); of 2048 11315 / 8303, 5719, 3521; 76 airfoils
-// of 300 335 / 348 (2); of 600 954 / 868 (2); of 1024 4802 / 3084 (2); 18 of 2048 14263
-// / 15700, 9393, 6006 (1, 2, 4).
+// block shape of k_ir_mixed / clusters): 1 airfoil of 200 panels 169 / 203, of 256 228 /
+// 257; 8 blocks: 1 of 300 319 / 303, of 600 794 / 586, of 1024 2677 / 1331, of 2048 8526 /
+// 3118; 4 blocks: 36 of 400 453 / 412, of 1024 3130 / 1721, of 2048 9863 / 5193; 2
+// blocks: 76 of 300 323 / 348, of 400 522 / 509, of 600 926 / 876, of 1024 3218 / 2651;
+// one block: 100 of 500 689 / 900, of 1024 3224 / 4005, so not taken.
 static int ir_cluster_blocks(const SolveArgs& a) {
   const int mv = a.bt.n_max + 1;
   if (a.ir_shape != 0 || mv <= kFuseM) return 0;
-  for (int C = 8; C >= 1; C >>= 1)
-    if (a.bt.B <= ir_cluster_capacity(C))
-      return ((C < 4 && mv <= 400) || (C == 1 && mv > 1400)) ? 0 : C;
+  for (int C = 8; C >= 2; C >>= 1)
+    if (a.bt.B <= ir_cluster_capacity(C)) return (C < 4 && mv <= 400) ? 0 : C;
   return 0;
 }
 
@@ -2046,6 +2045,9 @@ static cudaError_t launch_ir_kernel(const SolveArgs& a, cudaStream_t s) {
   // 3: 1 of 100 panels 90 / 87 / 85, 152 of 160 154 / 138 / 142, 304 of 200 283 / 279 /
   // 257, 608 of 256 644 / 790 / 702, 76 of 300 410 / 322 / 397)
   const int sms = sm_count(), mv = n_max + 1;
+  // (an airfoil per SM, 512 x 2 / 1024 x 1: 100 of 300 355 / 353, of 500 709 / 689, of
+  // 1024 3594 / 3224, forward system alone 2186 / 1996)
+  if (mv > 400 && a.bt.B <= sms) return launch_ir_shape<1024, 1>(a, s);
   if (fits(512, 2) && ((mv > 128 && a.bt.B <= sms) || (mv > kFuseM && a.bt.B <= 2 * sms)))
     return launch_ir_shape<512, 2>(a, s);
   if (mv <= kFuseM && a.bt.B <= 3 * sms) return launch_ir_shape<kThreads, 3>(a, s);
