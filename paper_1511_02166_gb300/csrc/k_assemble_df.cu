@@ -362,7 +362,8 @@ __global__ void __launch_bounds__(NT, MINB) k_assemble_df_tiles(
       const float Lj = pc[kL * ld + jl];
       const bool far_ji = gm.rho2.hi >= 16.0f * Li * Li;  // entry (j, i), panel i
       const bool far_ij = gm.rho2.hi >= 16.0f * Lj * Lj;  // entry (i, j), panel j
-      float th = __int_as_float(0x7fffffff), tl = 0.0f;  // NaN: a near-field entry
+      // a near-field entry: NaN with a low word of 0 (an evaluated NaN has both)
+      float th = __int_as_float(0x7fffffff), tl = 0.0f;
       if (__any_sync(0xffffffffu, far_ji || far_ij)) {
         const df2 X = df_sub(gm.px2, gm.py2);
         df2 Y = df_mul(gm.px, gm.py);
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(NT, MINB) k_assemble_df_tiles(
 #pragma unroll 4
     for (int q = lane / kTileRows; q < 32; q += 32 / kTileRows) {
       const float th = Th[q * kTileLd + jj], tl = Tl[q * kTileLd + jj];
-      if (jj < jn && i0 + 32 * ti + q < n && th == th) {
+      if (jj < jn && i0 + 32 * ti + q < n && (th == th || tl != tl)) {
         const int64_t e = (int64_t)(i0 + 32 * ti + q) * m + j0 + jb + jj;
         Ah[e] = th;
         Al[e] = tl;
