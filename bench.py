@@ -608,8 +608,7 @@ def measure_workload(name, mode, args, ctx, headline=False, extras=False):
     # the traffic row of the kernels in use: the factor's LU kernel as tuned
     tkey = dom
     if dom == "factor" and mode == "mixed":
-        kinds = {"lu" if bk["factor"] == "lu (shared memory)" else bk["factor"]
-                 for bk in pb.tuning()["buckets"]}
+        kinds = {bk["factor"] for bk in pb.tuning()["buckets"]}
         if len(kinds) == 1 and kinds != {"lu"}:
             tkey = "factor:" + kinds.pop()
     roof = {"kernel": dom, "bound": dk["bound"], "achieved": dk["achieved"], "peak": dk["peak"],

@@ -770,7 +770,7 @@ static size_t lu_global_smem(int n_max) {
 //            transposed: the previous group's columns of U^T (rows of U), or
 //            of L^T, applied to the rest of z, a thread per column
 //            (right-looking, coalesced across the threads); the group's own
-//            entries go to its 32-float scratch instead of z;
+//            entries go to its scratch (32 floats of 64) instead of z;
 //   phase B  the group's diagonal block: y_i = sum X_iq t_q, z_i = sum X_qi t_q
 //            (a few rows / columns per warp).
 // Solving both systems, every warp takes its share of both in each phase (the
