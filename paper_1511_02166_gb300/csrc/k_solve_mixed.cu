@@ -1885,11 +1885,11 @@ static SolveArgs make_args(const Batch& bt, const float* A_hi, const float* A_lo
 // Which one-block LU a launch of B airfoils of at most mv unknowns takes (1 through
 // L2, 2 in shared memory).  Up to 64 unknowns the shared-memory form's blocks of 128
 // threads, five on an SM, are the faster ones for any batch beyond three airfoils per
-// SM (4096 of 40 panels 145 us against 214; one 21 / 21).  Above, one to three of its
+// SM (4096 of 40 panels 138 us against 202; one 20 / 20).  Above, one to three of its
 // airfoils fit an SM and the L2-resident form is as fast or faster (4096 of 80 panels
-// 379 / 376, 128 1431 / 703, 205 2501 / 1557), but for a single airfoil per SM above
-// 160 unknowns, by its shorter steps (1 of 165 panels 69 / 72, of 205 91 / 98; 304 of
-// 165 141 / 93).  A launch that also holds larger airfoils runs them all through L2
+// 365 / 360, 128 1358 / 678, 205 2426 / 1526), but for a single airfoil per SM above
+// 160 unknowns, by its shorter steps (1 of 159 panels 57 / 54, of 160 65 / 68, of 205
+// 89 / 96; 304 of 165 133 / 89).  A launch that also holds larger airfoils runs them all through L2
 // at once.
 static int lu_kind_by_size(int B, int mv, int sms) {
   if (mv > kSmemLuM) return 1;
